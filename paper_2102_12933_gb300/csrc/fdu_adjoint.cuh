@@ -18,7 +18,7 @@ struct AdjEdgeArgs {
     double gm1, eps;
     // precision 48 (double-word edge VJP, fdu_adjoint_dw.cu)
     int prec;              // 64 or 48
-    const float2 *coefdw;  // [kEdgeCoef][ne] double-word coefficient block
+    const float4 *coefdw;  // [kDwPairs][ne] paired double-word coefficient block
     float dw_gm1[2], dw_tenth[2], dw_eps[2];
     int dw_eps_e;          // WENO epsilon = dw_eps * 2^dw_eps_e
 };

@@ -226,12 +226,17 @@ __device__ __forceinline__ WScale field_scale(dw a, dw b, dw c, dw d, dw e, dw f
 }
 
 // k: the 24 WENO coefficients of the edge (double words, global memory)
-__device__ __forceinline__ dw kc(const float2 *kp, int64_t ne, int i) {
-    const float2 q = __ldg(kp + (int64_t)i * ne);
-    return dw_make(q.x, q.y);
+__device__ __forceinline__ dw kc(const float4 *kp, int64_t ne, int i) {
+#pragma unroll
+    for (int p = 0; p < kDwPairs; ++p) {
+        const float4 q = __ldg(kp + (int64_t)p * ne);
+        if (dw_pair(p, 0) == i) return dw_make(q.x, q.z);
+        if (dw_pair(p, 1) == i) return dw_make(q.y, q.w);
+    }
+    return dw_make(0.0f);
 }
 
-__device__ __forceinline__ void weno_fwd_w(const float2 *kp, int64_t ne, dw a, dw b, dw c, dw d, dw e, dw f,
+__device__ __forceinline__ void weno_fwd_w(const float4 *kp, int64_t ne, dw a, dw b, dw c, dw d, dw e, dw f,
                                            dw eps_m, int eps_e, float2 *S, int fi) {
     const dw va = add_sl(mul_u(kc(kp, ne, 0), a), mul_u(kc(kp, ne, 1), b));
     const dw vb = add_sl(mul_u(kc(kp, ne, 5), b), mul_u(kc(kp, ne, 6), c));
@@ -281,7 +286,7 @@ __device__ __forceinline__ void weno_fwd_w(const float2 *kp, int64_t ne, dw a, d
 
 // Reverse of one field: from (dlb, drb) to the cotangents of a..f, written
 // over the field's forward slots as (a, b, c, d, e, f).
-__device__ __forceinline__ void weno_rev_w(const float2 *kp, int64_t ne, dw a, dw b, dw c, dw d, dw e, dw f, dw dlb,
+__device__ __forceinline__ void weno_rev_w(const float4 *kp, int64_t ne, dw a, dw b, dw c, dw d, dw e, dw f, dw dlb,
                                            dw drb, float2 *S, int fi) {
     const int w0 = kSlotW + 8 * fi;
     const dw va = ld_s(S, w0), vb = ld_s(S, w0 + 1), vc = ld_s(S, w0 + 2), vd = ld_s(S, w0 + 3);
@@ -344,7 +349,7 @@ __global__ void __launch_bounds__(kVjpBlock, 6) edge_flux_vjp_dw_kernel(AdjEdgeA
     float2 *S = stage + threadIdx.x;
     const double *__restrict__ w = A.w;
     const int64_t ne = A.ne;
-    const float2 *kp = A.coefdw + e;
+    const float4 *kp = A.coefdw + e;
     const dw gm1 = dw_make(A.dw_gm1[0], A.dw_gm1[1]);
     const dw eps_m = dw_make(A.dw_eps[0], A.dw_eps[1]);
     int32_t s[6];

@@ -64,7 +64,7 @@ struct fdu_mesh {
     // precision 48 (built on first use): double-word coefficient block
     // [kEdgeCoef][ne_act]; FP64 divergence tables with the left vertex flux
     // of each edge folded into the vertex weights; edge weights as double words
-    float2 *coefdw = nullptr;
+    float4 *coefdw = nullptr;
     double *swf48 = nullptr, *swg48 = nullptr, *cfg48 = nullptr;
     float2 *swe48 = nullptr;
     std::vector<int32_t> order64;     // vertex at each position of the FP64 SELL layout
@@ -438,16 +438,17 @@ fdu_status check_precision(fdu_mesh *m, int prec) {
     sell_tables(m, m->order64, wf.data(), wg.data(), T.we.data(), S);
     std::vector<float2> we2(S.we.size());
     for (size_t i = 0; i < we2.size(); ++i) we2[i] = split(S.we[i]);
-    std::vector<float2> k((size_t)kEdgeCoef * ne);
-    for (int64_t e = 0; e < ne; ++e) {
-        const int64_t o = T.e_new2old[e];
-        for (int c = 0; c < kEdgeCoef; ++c) k[(size_t)c * ne + e] = split(T.coef[(size_t)kEdgeCoef * o + c]);
-    }
     if ((st = m->upload(m->swf48, S.wf))) return st;
     if ((st = m->upload(m->swg48, S.wg))) return st;
     if ((st = m->upload(m->cfg48, cfg))) return st;
     if ((st = m->upload(m->swe48, we2))) return st;
-    return m->upload(m->coefdw, k);
+    float4 *k = nullptr;
+    if ((st = m->alloc(k, (size_t)kDwPairs * ne))) return st;
+    launch_coef_dw(m->coef64, k, ne, nullptr);
+    CK_LAUNCH();
+    CK(cudaDeviceSynchronize());
+    m->coefdw = k;
+    return FDU_OK;
 }
 
 // Double-word constants of the precision-48 edge flux.

@@ -15,74 +15,115 @@
 namespace fdu {
 namespace dwa {
 
-// ---- NU-WENO5 increments of one field, both sides (the block layout and
-// sub-stencil sharing of weno_pair64_l1; right increments from L1)
+// ---- NU-WENO5 increments of one field, both sides at once: lane 0 is the
+// left state, lane 1 the right (mirrored) one.  The right side's sub-stencils
+// are the left side's seen from R1, so every step of the two sides is the same
+// operation on paired operands: S_a with S_d, S_b with S_c (the sub-stencils
+// of weno_pair64_l1; right increments from L1).
+//   ae = (a, e) = (L3-L1, R3-R1), bf = (b, f) = (L2-L1, R2-R1), c = R1-L1,
+//   d = f + c = R2-L1 (characteristic components of one field)
+// K: the edge's paired coefficients (kDwPairs, fdu_internal.h).
 __device__ __forceinline__ int bexp(float x) { return (int)((__float_as_uint(x) >> 23) & 0xffu); }
+__device__ __forceinline__ f2 at_least(f2 x, float m) { return pk(fmaxf(lane0(x), m), fmaxf(lane1(x), m)); }
 
-__device__ __forceinline__ void weno_pair_dw(const dw *k, dw a, dw b, dw c, dw d, dw e, dw f, dw eps_m, int eps_e,
-                                             dw &dl, dw &dr) {
-    const dw va = add_sl(mul_u(k[0], a), mul_u(k[1], b));
-    const dw vb = add_sl(mul_u(k[5], b), mul_u(k[6], c));
-    const dw vc = add_sl(mul_u(k[10], c), mul_u(k[11], d));
-    const dw vd = add_sl(mul_u(k[15], e), mul_u(k[16], f));
-    const dw vdc = add_sl(vd, c);  // S_d's value from L1
+__device__ __forceinline__ dw2 weno_pair_dw(const dw2 *K, dw2 ae, dw2 bf, dw c, dw eps_m, int eps_e) {
+    const dw2 c1{pk(0.0f, c.h), pk(0.0f, c.l)}, cc = both(c);
+    const dw2 bd = norm(ladd(bf, c1));                                  // (b, d)
+    const dw2 v1 = norm(lfma(K[1], bf, lfma(K[0], ae, c1)));            // (v_a, v_d + c): S_d's value from L1
+    const dw2 v2 = norm(lfma(K[6], cc, lmul(K[5], bd)));                // (v_b, v_c)
     // common power-of-two scale of the six differences: max |.| in [1/2, 1)
-    const float mx = fmaxf(fmaxf(fmaxf(fabsf(a.h), fabsf(b.h)), fmaxf(fabsf(c.h), fabsf(d.h))),
-                           fmaxf(fabsf(e.h), fabsf(f.h)));
+    const float mx = fmaxf(fmaxf(fmaxf(fabsf(lane0(ae.h)), fabsf(lane1(ae.h))), fabsf(c.h)),
+                           fmaxf(fmaxf(fabsf(lane0(bf.h)), fabsf(lane1(bf.h))), fabsf(lane1(bd.h))));
     const int be = bexp(mx);
-    const int K = be == 0 ? 0 : be - 126;                  // mx in [2^(K-1), 2^K)
-    const float lam = __uint_as_float((unsigned)(127 - K) << 23);  // 2^-K (K in [-125, 128])
-    a = scale(a, lam);
-    b = scale(b, lam);
-    c = scale(c, lam);
-    d = scale(d, lam);
-    e = scale(e, lam);
-    f = scale(f, lam);
-    // eps 2^(-2K) = eps_m 2^(eps_e - 2K) (zero below the float range)
-    const int e2 = min(eps_e - 2 * K, 100) + 127;  // beyond 2^100 the weights are the linear ones anyway
-    const dw eps = e2 >= 1 ? scale(eps_m, __uint_as_float((unsigned)e2 << 23)) : dw_make(0.0f, 0.0f);
-    const dw b2 = mul_u(b, b), c2 = mul_u(c, c);
-    auto beta = [&](dw m0, dw m1, dw m2, dw xx, dw xy, dw yy) {
-        dw s = add_sl(add_sl(add_sl(mul_u(m0, xx), mul_u(m1, xy)), mul_u(m2, yy)), eps);
-        if (s.h < 0x1p-100f) s = dw_make(0x1p-100f, 0.0f);
-        return s;
-    };
-    const dw ra = recip(beta(k[2], k[3], k[4], mul_u(a, a), mul_u(a, b), b2));
-    const dw rb = recip(beta(k[7], k[8], k[9], b2, mul_u(b, c), c2));
-    const dw rc = recip(beta(k[12], k[13], k[14], c2, mul_u(c, d), mul_u(d, d)));
-    const dw rd = recip(beta(k[17], k[18], k[19], mul_u(e, e), mul_u(e, f), mul_u(f, f)));
+    const int Ke = be == 0 ? 0 : be - 126;                           // mx in [2^(Ke-1), 2^Ke)
+    const float lam = __uint_as_float((unsigned)(127 - Ke) << 23);  // 2^-Ke (Ke in [-125, 128])
+    const dw2 aes = lscale(ae, lam), bfs = lscale(bf, lam), bds = lscale(bd, lam);
+    const dw cs = lscale(c, lam);
+    // eps 2^(-2Ke) = eps_m 2^(eps_e - 2Ke) (zero below the float range)
+    const int e2 = min(eps_e - 2 * Ke, 100) + 127;  // beyond 2^100 the weights are the linear ones anyway
+    const dw2 eps = both(e2 >= 1 ? lscale(eps_m, __uint_as_float((unsigned)e2 << 23)) : dw_make(0.0f, 0.0f));
+    // beta + eps = x (m0 x + m1 y) + m2 y^2 + eps, held above 2^-100
+    const dw2 had = lfma(K[3], bfs, lmul(K[2], aes));
+    dw2 Bad = norm(lfma(aes, had, lfma(K[4], lmul(bfs, bfs), eps)));
+    const dw2 hbc = lfma(K[8], both(cs), lmul(K[7], bds));
+    dw2 Bbc = norm(lfma(bds, hbc, lfma(K[9], both(lmul(cs, cs)), eps)));
+    Bad.h = at_least(Bad.h, 0x1p-100f);
+    Bbc.h = at_least(Bbc.h, 0x1p-100f);
+    const dw2 r1 = lrecip(Bad), r2 = lrecip(Bbc), r3 = swapped(r2);
     // alpha_k = C_k / (beta_k + eps); the block stores C_0/C_1, C_2/C_1 (C_1 -> 1)
-    const dw l0 = mul(k[20], ra), l2 = mul(k[21], rc);
-    dl = mul(add_sl(add_sl(mul_u(l0, va), mul_u(rb, vb)), mul_u(l2, vc)), recip(add_sl(add_sl(l0, rb), l2)));
-    const dw r0 = mul(k[22], rd), r2 = mul(k[23], rb);
-    dr = mul(add_sl(add_sl(mul_u(r0, vdc), mul_u(rc, vc)), mul_u(r2, vb)), recip(add_sl(add_sl(r0, rc), r2)));
+    const dw2 l0 = lmul(K[10], r1), l2 = lmul(K[11], r3);
+    const dw2 num = norm(lfma(l2, swapped(v2), lfma(r2, v2, lmul(l0, v1))));
+    return norm(lmul(num, norm(lrecip(norm(ladd(ladd(l0, r2), l2))))));
 }
 
-// ---- the edge flux
-// Per-thread staging in shared memory, slot j of thread t at [j][t]: the
-// five differences (slots 0-19, projected in place) and the WENO
-// increments (20-27).  The projections and the four fields run as loops
-// over the staged values, so their code is issued from the instruction
-// cache once per loop instead of being unrolled five and four times.
-constexpr int kDwSlots = 28;
+// ---- the edge flux, in the edge's frame: a state's momentum is kept as its
+// components along the normal n and the tangent t = (-n_y, n_x), which the
+// flux along the edge does not mix, and the result is turned back at the end.
+// Against x-y components this drops the two direction products from every
+// projection, back-projection, Roe average and flux.
+// A 4-vector (rho, m_n, m_t, rho E) or (fields q_n - c, entropy, shear, q_n + c).
+template <class T>
+struct vec4 {
+    dwv<T> x, n, t, w;
+};
+struct RoeN {  // Roe average along the edge: q_n, q_t, H, c, (q_n^2 + q_t^2)/2, (gamma-1)/(2c^2), 1/(2c)
+    dw q, t, H, c, hq2, b1h, ich;
+};
+__device__ __forceinline__ RoeN roe_n(dw q, dw t, dw H, dw gm1) {
+    RoeN R;
+    R.q = q;
+    R.t = t;
+    R.H = norm(H);
+    R.hq2 = norm(lscale(lfma(t, t, lmul(q, q)), 0.5f));
+    const dw c2 = norm(lmul(gm1, norm(lsub(R.H, R.hq2))));
+    const dw ic = norm(lrsqrt(c2));
+    R.c = norm(lmul(c2, ic));
+    R.b1h = norm(lscale(lmul(gm1, lmul(ic, ic)), 0.5f));
+    R.ich = lscale(ic, 0.5f);
+    return R;
+}
+__device__ __forceinline__ dw bcast(dw x, float) { return x; }
+__device__ __forceinline__ dw2 bcast(dw x, f2) { return both(x); }
+#define FDU_B(x) bcast(x, T{})
+template <class T>
+__device__ __forceinline__ vec4<T> project_n(const RoeN &R, const vec4<T> &d) {
+    const dwv<T> q = FDU_B(R.q), t = FDU_B(R.t);
+    const dwv<T> phh = lmul(FDU_B(R.b1h), lfma(lneg(t), d.t, lfma(lneg(q), d.n, lfma(FDU_B(R.hq2), d.x, d.w))));
+    const dwv<T> psh = lmul(FDU_B(R.ich), lfma(q, d.x, lneg(d.n)));
+    return vec4<T>{ladd(phh, psh), lsub(d.x, lscale(phh, 2.0f)), lfma(lneg(t), d.x, d.t), lsub(phh, psh)};
+}
+template <class T>
+__device__ __forceinline__ vec4<T> unproject_n(const RoeN &R, const vec4<T> &c) {
+    const dwv<T> q = FDU_B(R.q), t = FDU_B(R.t);
+    const dwv<T> ac = ladd(c.x, c.w), rho = ladd(ac, c.n), dd = lmul(FDU_B(R.c), lsub(c.w, c.x));
+    return vec4<T>{rho, lfma(q, rho, dd), lfma(t, rho, c.t),
+                   lfma(t, c.t, lfma(q, dd, lfma(FDU_B(R.hq2), c.n, lmul(FDU_B(R.H), ac))))};
+}
+// (x, y) momentum components to (n, t) ones
+template <class T>
+__device__ __forceinline__ void turn(dw nx, dw ny, dwv<T> mx, dwv<T> my, dwv<T> &n, dwv<T> &t) {
+    const dwv<T> a = FDU_B(nx), b = FDU_B(ny);
+    n = lfma(b, my, lmul(a, mx));
+    t = lfma(lneg(b), mx, lmul(a, my));
+}
+
+// Per-thread staging in shared memory, 16-byte slot j of thread t at [j][t]:
+// the four fields' (b, f), (a, e) and, two to a slot, c; the increments (dl,
+// dr) take the (b, f) slots.  The fields run as a loop over the staged values:
+// unrolled by two or four the kernel is slower (0.1167 and 0.137 ms against
+// 0.1146 ms at 250k vertices), its code then overflows the instruction caches.
+constexpr int kDwSlots = 10;
 // slot j of a thread at S[j * stride] (stride = the threads of the block)
 struct Stage {
-    float2 *S;
+    float4 *S;
     int stride;
 };
-__device__ __forceinline__ void st_dw(const Stage &T, int j, dw v) { T.S[j * T.stride] = make_float2(v.h, v.l); }
-__device__ __forceinline__ dw ld_dw(const Stage &T, int j) {
-    const float2 q = T.S[j * T.stride];
-    return dw_make(q.x, q.y);
+__device__ __forceinline__ void st_dw2(const Stage &T, int j, dw2 v) {
+    T.S[j * T.stride] = make_float4(lane0(v.h), lane1(v.h), lane0(v.l), lane1(v.l));
 }
-__device__ __forceinline__ void st_dw4(const Stage &S, int j, const dw4 &v) {
-    st_dw(S, j, v.x);
-    st_dw(S, j + 1, v.y);
-    st_dw(S, j + 2, v.z);
-    st_dw(S, j + 3, v.w);
-}
-__device__ __forceinline__ dw4 ld_dw4(const Stage &S, int j) {
-    return d4(ld_dw(S, j), ld_dw(S, j + 1), ld_dw(S, j + 2), ld_dw(S, j + 3));
+__device__ __forceinline__ dw2 ld_dw2(const Stage &T, int j) {
+    const float4 q = T.S[j * T.stride];
+    return dw2{pk(q.x, q.y), pk(q.z, q.w)};
 }
 
 __device__ __forceinline__ void edge_flux_dw_body(const EdgeArgs &A, const int64_t e, const Stage &S) {
@@ -92,122 +133,162 @@ __device__ __forceinline__ void edge_flux_dw_body(const EdgeArgs &A, const int64
     int32_t s[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) s[i] = __ldg(A.sten + (int64_t)i * ne + e);
-    const float2 nq = __ldg(A.coefdw + (int64_t)kCoefN * ne + e), mq = __ldg(A.coefdw + (int64_t)(kCoefN + 1) * ne + e);
-    const dw nx = dw_make(nq.x, nq.y), ny = dw_make(mq.x, mq.y);
-    const d4v L1 = ldd4(w, s[2]);
-    dw4 b;  // L1 in double words
-    {
-        // FP64 differences, then double words: R1-L1, L2-L1, L3-L1, R2-R1, R3-R1
-        auto diff = [](const d4v &p, const d4v &q) { return d2dw4(d4v{p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w}); };
-        const d4v R1 = ldd4(w, s[3]);
-        st_dw4(S, 0, diff(R1, L1));
-        st_dw4(S, 4, diff(ldd4(w, s[1]), L1));
-        st_dw4(S, 8, diff(ldd4(w, s[0]), L1));
-        st_dw4(S, 12, diff(ldd4(w, s[4]), R1));
-        st_dw4(S, 16, diff(ldd4(w, s[5]), R1));
-        b = d2dw4(L1);
-    }
-    const RoeW C = roe_records(d2dw4(ldd4(A.Q, s[2])), d2dw4(ldd4(A.Q, s[3])), nx, ny, gm1);
-#pragma unroll 1
-    for (int j = 0; j < 20; j += 4) st_dw4(S, j, project(C, ld_dw4(S, j)));
+    const float4 nq = __ldg(A.coefdw + (int64_t)(kDwPairs - 1) * ne + e);
+    const dw nx = dw_make(nq.x, nq.z), ny = dw_make(nq.y, nq.w);
 
+    // Roe average of the end states from their records (the two summed in FP64)
+    RoeN C;
     {
-        dw k[kCoefN];
+        const d4v qa = ldd4(A.Q, s[2]), qb = ldd4(A.Q, s[3]);
+        const dw4 q = d2dw4(d4v{qa.x + qb.x, qa.y + qb.y, qa.z + qb.z, qa.w + qb.w});
+        const dw inv = norm(lrecip(q.x));
+        dw mn, mt;
+        turn(nx, ny, q.y, q.z, mn, mt);
+        C = roe_n(norm(lmul(mn, inv)), norm(lmul(mt, inv)), lmul(q.w, inv), gm1);
+    }
+    vec4<float> b;  // L1
+    {
+        // FP64 differences, then double words in the edge's frame and their
+        // characteristic components: (L2-L1, R2-R1) and (L3-L1, R3-R1) paired, R1-L1
+        const d4v L1 = ldd4(w, s[2]), R1 = ldd4(w, s[3]);
+        auto diff = [](const d4v &p, const d4v &q) { return d2dw4(d4v{p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w}); };
+        auto two = [&](int il, int ir, int slot) {
+            const dw4 l = diff(ldd4(w, il), L1), r = diff(ldd4(w, ir), R1);
+            vec4<f2> d;
+            d.x = pair(l.x, r.x);
+            d.w = pair(l.w, r.w);
+            turn(nx, ny, pair(l.y, r.y), pair(l.z, r.z), d.n, d.t);
+            const vec4<f2> c = project_n(C, d);
+            st_dw2(S, slot, norm(c.x));
+            st_dw2(S, slot + 1, norm(c.n));
+            st_dw2(S, slot + 2, norm(c.t));
+            st_dw2(S, slot + 3, norm(c.w));
+        };
+        two(s[1], s[4], 0);
+        two(s[0], s[5], 4);
+        const dw4 m = diff(R1, L1), l = d2dw4(L1);
+        vec4<float> d;
+        d.x = m.x;
+        d.w = m.w;
+        turn(nx, ny, m.y, m.z, d.n, d.t);
+        const vec4<float> c = project_n(C, d);
+        st_dw2(S, 8, norm(pair(c.x, c.n)));
+        st_dw2(S, 9, norm(pair(c.t, c.w)));
+        b.x = l.x;
+        b.w = l.w;
+        turn(nx, ny, l.y, l.z, b.n, b.t);
+        b.n = norm(b.n);
+        b.t = norm(b.t);
+    }
+    {
+        dw2 K[kDwPairs - 1];
 #pragma unroll
-        for (int i = 0; i < kCoefN; ++i) {
-            const float2 q = __ldg(A.coefdw + (int64_t)i * ne + e);
-            k[i] = dw_make(q.x, q.y);
+        for (int i = 0; i < kDwPairs - 1; ++i) {
+            const float4 q = __ldg(A.coefdw + (int64_t)i * ne + e);
+            K[i] = dw2{pk(q.x, q.y), pk(q.z, q.w)};
         }
         const dw eps_m = dw_make(A.dw_eps[0], A.dw_eps[1]);
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) {
-            const dw c = ld_dw(S, i), f = ld_dw(S, 12 + i);
-            dw dl, dr;
-            weno_pair_dw(k, ld_dw(S, 8 + i), ld_dw(S, 4 + i), c, add_sl(f, c), ld_dw(S, 16 + i), f, eps_m, A.dw_eps_e,
-                         dl, dr);
-            st_dw(S, 20 + i, dl);
-            st_dw(S, 24 + i, dr);
+            const dw2 cq = ld_dw2(S, 8 + (i >> 1));
+            st_dw2(S, i, weno_pair_dw(K, ld_dw2(S, 4 + i), ld_dw2(S, i), (i & 1) ? second(cq) : first(cq), eps_m,
+                                      A.dw_eps_e));
         }
     }
 
-    // increments of both interpolated states from L1
-    dw4 il = unproject(C, ld_dw4(S, 20)), ir = unproject(C, ld_dw4(S, 24));
-
     // primitives of L1
-    const dw ib = recip(b.x);
-    const dw ub = mul(b.y, ib), vb = mul(b.z, ib);
-    const dw qnb = add_sl(mul_u(ub, nx), mul_u(vb, ny));
-    const dw mu = add_sl(mul_u(b.y, ub), mul_u(b.z, vb));  // |m|^2 / rho
-    const dw pb = mul(gm1, sub_sl(b.w, scale(mu, 0.5f)));
+    const dw ib = norm(lrecip(b.x));
+    const dw qnb = norm(lmul(b.n, ib)), qtb = norm(lmul(b.t, ib));
+    const dw mu = lfma(b.t, qtb, lmul(b.n, qnb));  // |m|^2 / rho
+    const dw pb = norm(lmul(gm1, lsub(b.w, lscale(mu, 0.5f))));
 
-    // a side's state from its increment: rho', 1/sqrt(rho'), the normal
-    // velocity increment and the pressure increment
-    struct Side {
-        dw rho, r, ir, dq, dp, p;
-    };
-    auto side = [&](const dw4 &dd, Side &Sd) {
-        Sd.rho = add_sl(b.x, dd.x);
-        if (!(Sd.rho.h > 0.0f)) return false;
-        Sd.r = rsqrt(Sd.rho);
-        Sd.ir = mul(Sd.r, Sd.r);
-        Sd.dq = mul(sub_sl(add_sl(mul_u(dd.y, nx), mul_u(dd.z, ny)), mul_u(qnb, dd.x)), Sd.ir);
+    // increments of both interpolated states (left, right) from L1
+    vec4<f2> dd = unproject_n(C, vec4<f2>{ld_dw2(S, 0), ld_dw2(S, 1), ld_dw2(S, 2), ld_dw2(S, 3)});
+    dd = vec4<f2>{norm(dd.x), norm(dd.n), norm(dd.t), norm(dd.w)};
+    // the states from their increments: rho', 1/sqrt(rho'), the normal velocity
+    // and pressure increments
+    struct Sides {
+        dw2 rho, r, dq, dp, p;
+    } P;
+    auto sides = [&]() {
+        P.rho = norm(ladd(both(b.x), dd.x));
+        if (!(lane0(P.rho.h) > 0.0f && lane1(P.rho.h) > 0.0f)) return false;
+        P.r = norm(lrsqrt(P.rho));
+        const dw2 ir = norm(lmul(P.r, P.r));
+        P.dq = norm(lmul(lfma(both(lneg(qnb)), dd.x, dd.n), ir));
         // K' - K = ((2m + dm).dm - (|m|^2/rho) drho) / (2 rho')
-        const dw t = sub_sl(add_sl(mul_u(add_sl(scale(b.y, 2.0f), dd.y), dd.y),
-                                   mul_u(add_sl(scale(b.z, 2.0f), dd.z), dd.z)),
-                            mul_u(mu, dd.x));
-        Sd.dp = mul(gm1, sub_sl(dd.w, scale(mul(t, Sd.ir), 0.5f)));
-        Sd.p = add_sl(pb, Sd.dp);
-        return Sd.p.h > 0.0f;
+        const dw2 k2 = lfma(both(lneg(mu)), dd.x,
+                            lfma(ladd(both(lscale(b.t, 2.0f)), dd.t), dd.t,
+                                 lmul(ladd(both(lscale(b.n, 2.0f)), dd.n), dd.n)));
+        P.dp = lmul(both(gm1), lfma(lscale(k2, -0.5f), ir, dd.w));
+        P.p = norm(ladd(both(pb), P.dp));
+        return lane0(P.p.h) > 0.0f && lane1(P.p.h) > 0.0f;
     };
-    Side SL, SR;
-    bool ok = side(il, SL);
-    ok = ok && side(ir, SR);
-    if (!ok) {  // positivity fallback: first-order end states
-        const d4v R1 = ldd4(w, s[3]);
-        il = d4(dw_make(0.0f), dw_make(0.0f), dw_make(0.0f), dw_make(0.0f));
-        ir = d2dw4(d4v{R1.x - L1.x, R1.y - L1.y, R1.z - L1.z, R1.w - L1.w});
-        side(il, SL);
-        side(ir, SR);
+    if (!sides()) {  // positivity fallback: first-order end states
+        const d4v L1 = ldd4(w, s[2]), R1 = ldd4(w, s[3]);
+        const dw4 m = d2dw4(d4v{R1.x - L1.x, R1.y - L1.y, R1.z - L1.z, R1.w - L1.w});
+        const dw z = dw_make(0.0f);
+        dw n, t;
+        turn(nx, ny, m.y, m.z, n, t);
+        dd = vec4<f2>{pair(z, m.x), pair(z, n), pair(z, t), pair(z, m.w)};
+        sides();
         atomicAdd(A.fallback, 1ull);
     }
 
     // flux increment F_n(w_L) - F_n(L1)
-    const dw qnl = add_sl(qnb, SL.dq);
-    dw4 out;
-    out.x = add_sl(mul_u(il.y, nx), mul_u(il.z, ny));
-    out.y = add_sl(add_sl(mul_u(il.y, qnl), mul_u(b.y, SL.dq)), mul_u(SL.dp, nx));
-    out.z = add_sl(add_sl(mul_u(il.z, qnl), mul_u(b.z, SL.dq)), mul_u(SL.dp, ny));
-    out.w = add_sl(mul_u(add_sl(il.w, SL.dp), qnl), mul_u(add_sl(b.w, pb), SL.dq));
+    const vec4<float> il{first(dd.x), first(dd.n), first(dd.t), first(dd.w)};
+    const dw dql = first(P.dq), dpl = first(P.dp);
+    const dw qnl = norm(ladd(qnb, dql));
+    vec4<float> out;
+    out.x = il.n;
+    out.n = lfma(b.n, dql, lfma(il.n, qnl, dpl));
+    out.t = lfma(b.t, dql, lmul(il.t, qnl));
+    out.w = lfma(ladd(b.w, pb), dql, lmul(ladd(il.w, dpl), qnl));
 
     // Roe dissipation at the Roe average of (w_L, w_R)
     {
-        const dw4 wl = add4_sl(b, il), wr = add4_sl(b, ir);
-        const dw sa = mul_u(SL.rho, SL.r), sb = mul_u(SR.rho, SR.r);
-        const dw inv = recip(add_sl(sa, sb));
-        const RoeW Q = roe_finish(mul(add_sl(mul_u(wl.y, SL.r), mul_u(wr.y, SR.r)), inv),
-                                  mul(add_sl(mul_u(wl.z, SL.r), mul_u(wr.z, SR.r)), inv),
-                                  mul(add_sl(mul_u(add_sl(wl.w, SL.p), SL.r), mul_u(add_sl(wr.w, SR.p), SR.r)), inv),
-                                  nx, ny, gm1);
-        const dw4 a = project(Q, sub4_sl(ir, il));
-        const dw delta = mul(Q.c, dw_make(A.dw_tenth[0], A.dw_tenth[1]));
-        const dw h2d = mul(Q.ic, 5.0f);  // 1 / (2 delta)
-        auto negp = [&](dw l) {  // (l - |l|_fixed) / 2
-            const dw m = dabs(l);
-            if (m.h < delta.h || (m.h == delta.h && m.l < delta.l))
-                return scale(sub_sl(l, mul(add_sl(mul_u(l, l), mul_u(delta, delta)), h2d)), 0.5f);
-            return l.h < 0.0f ? l : dw_make(0.0f);
+        const dw2 sr = lmul(P.rho, P.r);
+        const dw inv = norm(lrecip(ladd(first(sr), second(sr))));
+        auto avg = [&](dw2 x) {
+            const dw2 y = lmul(x, P.r);
+            return lmul(ladd(first(y), second(y)), inv);
         };
-        const dw nu = negp(Q.qn), nm = negp(sub_sl(Q.qn, Q.c)), np = negp(add_sl(Q.qn, Q.c));
-        const dw4 D = unproject(Q, d4(mul(nm, a.x), mul(nu, a.y), mul(nu, a.z), mul(np, a.w)));
-        out = add4_sl(out, D);
+        const RoeN Q = roe_n(norm(avg(ladd(both(b.n), dd.n))), norm(avg(ladd(both(b.t), dd.t))),
+                             avg(ladd(ladd(both(b.w), dd.w), P.p)), gm1);
+        const vec4<float> a = project_n(Q, vec4<float>{lsub(second(dd.x), il.x), lsub(second(dd.n), il.n),
+                                                       lsub(second(dd.t), il.t), lsub(second(dd.w), il.w)});
+        // (l - |l|_fixed) / 2: min(l, 0), or -(l - delta)^2 / (4 delta) inside Harten's band |l| < delta = 0.1 c
+        const dw delta = norm(lmul(Q.c, dw_make(A.dw_tenth[0], A.dw_tenth[1])));
+        const dw h4d = norm(lmul(Q.ich, dw_make(5.0f)));  // 1 / (4 delta)
+        auto fixed = [&](float lh, float ll, float fh, float fl) {
+            const float ah = fabsf(lh), al = lh < 0.0f ? -ll : ll;
+            const bool in = ah < delta.h || (ah == delta.h && al < delta.l);
+            const bool up = !(lh < 0.0f);
+            return dw_make(in ? -fh : up ? 0.0f : lh, in ? -fl : up ? 0.0f : ll);
+        };
+        const dw2 lmp = norm(ladd(both(Q.q), pair(lneg(Q.c), Q.c)));  // q_n - c, q_n + c
+        const dw2 smp = norm(lsub(lmp, both(delta)));
+        const dw2 fmp = norm(lmul(lmul(smp, smp), both(h4d)));
+        const dw su = norm(lsub(Q.q, delta)), fu = norm(lmul(lmul(su, su), h4d));
+        const dw nm = fixed(lane0(lmp.h), lane0(lmp.l), lane0(fmp.h), lane0(fmp.l));
+        const dw np = fixed(lane1(lmp.h), lane1(lmp.l), lane1(fmp.h), lane1(fmp.l));
+        const dw nu = fixed(Q.q.h, Q.q.l, fu.h, fu.l);
+        const vec4<float> D = unproject_n(Q, vec4<float>{lmul(nm, a.x), lmul(nu, a.n), lmul(nu, a.t), lmul(np, a.w)});
+        out.x = ladd(out.x, D.x);
+        out.n = ladd(out.n, D.n);
+        out.t = ladd(out.t, D.t);
+        out.w = ladd(out.w, D.w);
     }
 
-    // the increment r - F_n(L1); the divergence adds F_n(L1) through its
-    // folded vertex weights
+    // the increment r - F_n(L1), back in x-y components; the divergence adds
+    // F_n(L1) through its folded vertex weights
+    const dw2 m = norm(lfma(pair(lneg(ny), nx), both(out.t), lmul(pair(nx, ny), both(out.n))));
+    const dw2 xw = norm(pair(out.x, out.w));
     float4 *r = static_cast<float4 *>(A.r);
-    r[2 * e] = make_float4(out.x.h, out.x.l, out.y.h, out.y.l);
-    r[2 * e + 1] = make_float4(out.z.h, out.z.l, out.w.h, out.w.l);
+    r[2 * e] = make_float4(lane0(xw.h), lane0(xw.l), lane0(m.h), lane0(m.l));
+    r[2 * e + 1] = make_float4(lane1(m.h), lane1(m.l), lane1(xw.h), lane1(xw.l));
 }
+#undef FDU_B
 
 }  // namespace dwa
 }  // namespace fdu

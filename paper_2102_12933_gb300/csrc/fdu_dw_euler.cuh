@@ -7,9 +7,17 @@
 #include <cstdint>
 
 #include "fdu_dw.cuh"
+#include "fdu_internal.h"
 
 namespace fdu {
 namespace dwa {
+
+// Values (of the kEdgeCoef block) in lane 0 and 1 of pair p of the paired block.
+__device__ constexpr int dw_pair(int p, int lane) {
+    constexpr int t[kDwPairs][2] = {{0, 15}, {1, 16}, {2, 17}, {3, 18}, {4, 19},   {5, 11},  {6, 10},
+                                    {7, 14}, {8, 13}, {9, 12}, {20, 22}, {21, 23}, {kCoefN, kCoefN + 1}};
+    return t[p][lane];
+}
 
 struct dw4 {
     dw x, y, z, w;
@@ -53,12 +61,6 @@ __device__ __forceinline__ RoeW roe_finish(dw u, dw v, dw H, dw nx, dw ny, dw gm
     R.qn = add_sl(mul_u(u, nx), mul_u(v, ny));
     R.qt = sub_sl(mul_u(v, nx), mul_u(u, ny));
     return R;
-}
-// Roe average from the sides' records (sqrt rho, sqrt rho u, sqrt rho v, sqrt rho H)
-__device__ __forceinline__ RoeW roe_records(const dw4 &qa, const dw4 &qb, dw nx, dw ny, dw gm1) {
-    const dw inv = recip(add_sl(qa.x, qb.x));
-    return roe_finish(mul(add_sl(qa.y, qb.y), inv), mul(add_sl(qa.z, qb.z), inv), mul(add_sl(qa.w, qb.w), inv), nx,
-                      ny, gm1);
 }
 // fields q_n - c, q_n (entropy), q_n (shear), q_n + c
 // Sums of increments (here and in the WENO values and weighted sums) take

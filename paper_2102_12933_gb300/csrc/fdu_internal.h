@@ -34,6 +34,12 @@ constexpr int kCoefCL = 20;
 constexpr int kCoefCR = 22;
 constexpr int kCoefN = 24;
 constexpr int kEdgeCoef = 26;
+// Precision 48: the block as double words, paired for the kernels that work on
+// the left and right states in the two lanes of packed FP32 instructions: pair
+// i of an edge is one float4 (first.h, second.h, first.l, second.l), [kDwPairs]
+// [ne].  The pairs put S_a's values beside S_d's and S_b's beside the mirrored
+// S_c's (dw_pair, fdu_dw_euler.cuh); the last is the normal.
+constexpr int kDwPairs = 13;
 // FP32 path, default form: the FP64-built block rounded to FP32, values
 // 0..23 as six float4 per edge ([6][ne] float4, value c at block c / 4,
 // component c % 4), then (n_x, n_y) as one float2 per edge ([ne] float2

@@ -802,14 +802,14 @@ __global__ void stage_persistent_kernel(EdgeArgs EA, DivArgs DA, unsigned int *b
 }
 
 // Precision 48: the same stage with the double-word edge flux (its staging in
-// dynamic shared memory, kDwSlots double words per thread) and the folded
+// dynamic shared memory, kDwSlots 16-byte slots per thread) and the folded
 // divergence.  At most 512 threads a block, so at most 128 registers.
 template <int MODE>
 __global__ void __launch_bounds__(512, 1)
     stage_persistent_dw_kernel(EdgeArgs EA, DivArgs DA, unsigned int *bar_count, unsigned int *bar_gen,
                                unsigned int nblocks_expected, unsigned long long spin_limit, int *err) {
     if (barrier_failed(err)) return;
-    extern __shared__ float2 dw_stage[];
+    extern __shared__ float4 dw_stage[];
     const dwa::Stage T{dw_stage + threadIdx.x, (int)blockDim.x};
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1012,7 +1012,7 @@ cudaError_t coop(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigne
 }  // namespace
 
 namespace {
-size_t dw_stage_bytes(int threads) { return (size_t)dwa::kDwSlots * sizeof(float2) * threads; }
+size_t dw_stage_bytes(int threads) { return (size_t)dwa::kDwSlots * sizeof(float4) * threads; }
 template <int MODE>
 cudaError_t coop48(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigned int *g, unsigned int ne,
                    unsigned long long lim, int *err, int threads, int nb, cudaStream_t s) {

@@ -28,7 +28,7 @@ struct EdgeArgs {
     // double-word edge flux (precision 48; Q is required there): r receives
     // the increment r_k - F_n(L1_k) as double words, [ne] x two float4
     // (h0, l0, h1, l1), (h2, l2, h3, l3)
-    const float2 *coefdw; // [kEdgeCoef][ne] (hi, lo) of the coefficient block
+    const float4 *coefdw; // [kDwPairs][ne] paired double words of the coefficient block
     float dw_gm1[2];      // gamma - 1 as a double word
     float dw_tenth[2];    // 0.1 as a double word
     float dw_eps[2];      // WENO epsilon = dw_eps * 2^dw_eps_e, dw_eps in [1, 2)
@@ -75,6 +75,8 @@ void launch_vertex_flux_f32(const double *w, float4 *F, float4 *w32, int64_t n, 
 void launch_edge_flux_f64(const EdgeArgs &a, cudaStream_t s);
 void launch_edge_flux_f32(const EdgeArgs &a, cudaStream_t s);
 void launch_edge_flux_dw(const EdgeArgs &a, cudaStream_t s);
+// coefdw[kDwPairs][ne] = the double words of coef[kEdgeCoef][ne], paired
+void launch_coef_dw(const double *coef, float4 *coefdw, int64_t ne, cudaStream_t s);
 // z = double-word primitive `op` of x (and y), device pointers (accuracy check)
 void launch_dw_check(int op, const double *x, const double *y, double *z, int64_t n, cudaStream_t s);
 void launch_div_f64(const DivArgs &a, int mode, cudaStream_t s);
