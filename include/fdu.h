@@ -182,16 +182,18 @@ fdu_status fdu_get_state(const fdu_mesh *mesh, double *w, int on_device, void *s
 
 /* Spatial residual dwdt[nv][4] = -(a1 + b2) per component of the current
  * state (Section 2.2.1), with edge fluxes from characteristic NU-WENO5
- * and a Roe flux (Section 2.3.1, Appendix).  precision = 64 computes in
- * FP64; precision = 32 reads FP32 copies of the state and tables and
- * computes in FP32; precision = 48 is the FP64 computation with the edge
- * flux's increments (characteristic projection, WENO, flux increment and
- * Roe dissipation) in double-word FP32 arithmetic (FP32 pairs, about 48
- * significant bits) and its state-sized terms (stencil differences, the
- * vertex flux at the edge's left end, the final sum) in FP64: the same
- * function to the FP64 path's tolerance, faster on parts whose FP64 rate
- * is a small fraction of their FP32 rate.  Its first use builds a
- * double-word copy of the edge coefficient block (192 bytes per edge).
+ * and a Roe flux (Section 2.3.1, Appendix).  precision = 32 reads FP32
+ * copies of the state and tables and computes in FP32.  precision = 64 has
+ * FP64 accuracy: state-sized terms (stencil differences, vertex fluxes and
+ * their weighted sums, the stage update) are FP64, and the edge flux's
+ * increments (characteristic projection, WENO, flux increment, Roe
+ * dissipation) are double-word FP32 (FP32 pairs, about 48 significant bits),
+ * which GB300 issues at 64 times its FP64 rate and whose error in the
+ * residual is no larger than that of the same sums taken in FP64 throughout.
+ * Where FP32 pairs would not do, it computes in FP64 throughout: a stage with
+ * a density or energy outside 2^-24 .. 2^24 (in the caller's units), a mesh
+ * with weights beyond 2^40, and single edges beyond Mach 3.9.  precision = 48
+ * is the double-word path without these checks.
  * Ghost vertices get 0.  With on_device = 0 the call synchronises `stream`
  * before returning.  The RK calls below accept the same three values. */
 fdu_status fdu_residual(fdu_mesh *mesh, int precision, double *dwdt, int on_device, void *stream);

@@ -61,13 +61,14 @@ struct fdu_mesh {
     int32_t *sten = nullptr;          // [6][ne_act]
     double *coef64 = nullptr;         // [32][ne_act]
     float *coef32 = nullptr;          // FP32 block: [6][ne_act] float4, or (f32_coef = 1) [ne_act] float4 of gaps; then [ne_act] float2 (n_x, n_y)
-    // precision 48 (built on first use): double-word coefficient block
-    // [kEdgeCoef][ne_act]; FP64 divergence tables with the left vertex flux
-    // of each edge folded into the vertex weights; edge weights as double words
+    // precisions 64 and 48: paired double-word coefficient block [kDwPairs]
+    // [ne_act]; FP64 divergence tables with the left vertex flux of each edge
+    // folded into the vertex weights; edge weights as double words
     float4 *coefdw = nullptr;
     double *swf48 = nullptr, *swg48 = nullptr, *cfg48 = nullptr;
     float2 *swe48 = nullptr;
-    std::vector<int32_t> order64;     // vertex at each position of the FP64 SELL layout
+    bool fold_ok = false;             // the folded tables hold (precision 48 is available)
+    bool dw64 = false;                // precision 64 takes the double-word path (fold_ok, tables in its window)
     int64_t *slice_voff = nullptr, *slice_eoff = nullptr;       // FP32 layout (natural order)
     int64_t *slice_voff64 = nullptr, *slice_eoff64 = nullptr;   // FP64 layout (stencil-size order in windows)
     int32_t *svid64 = nullptr, *seid64 = nullptr, *perm64 = nullptr;
@@ -85,10 +86,14 @@ struct fdu_mesh {
     float4 *w32 = nullptr;                                  // [nv]
     double *r64 = nullptr;                                  // [ne_act][4]
     float4 *r32 = nullptr;                                  // [ne_act]
-    unsigned long long *counters = nullptr;  // [0] fallbacks, [1] dt slot, [2] adaptive slot, [3] adaptive steps,
+    unsigned long long *counters = nullptr;  // [0] fallbacks, [1] dt slot, [2] adaptive slot, [3] unused,
                                              // [4] stage updates scaled by the positivity safeguard,
                                              // [5] first non-physical row of a state being set
-    double *tstate = nullptr;                // adaptive stepping: (t, dt, nonphysical flag)
+    // adaptive stepping: (t, dt, nonphysical flag), then the step counter and
+    // the wide flags in the fourth to sixth words, all reset by one memset
+    double *tstate = nullptr;
+    unsigned long long *nsteps = nullptr;    // adaptive steps taken (in tstate's fourth word)
+    int *wide = nullptr;                     // [kWideSlots] (in tstate's fifth and sixth words)
     bool f64_valid = false, f32_valid = false;              // F64[0] / (w32, F32[0]) describe wn
     cudaStream_t own_stream = nullptr;
     std::map<std::pair<int, double>, cudaGraphExec_t> graphs;
@@ -239,6 +244,46 @@ void stencil_gaps(const double xi[6], float g[4]) {
     for (int c = 0; c < 4; ++c) g[c] = (float)d[c];
 }
 
+// The double-word tables of precisions 64 and 48, formed on the device from the
+// FP64 tables (on the host this took 0.2 s at 250k vertices, here a
+// millisecond):
+//  - the double-word edge coefficient block (hi = the FP32 rounding of each
+//    FP64 coefficient, lo = the FP32 rounding of the remainder);
+//  - divergence tables in the FP64 SELL layout where the edge flux, which
+//    the double-word edge kernel leaves as the increment
+//    r_k - F_n(L1_k) = r_k - (n_x f + n_y g)(L1_k), has its left-vertex part
+//    folded into the weights of that vertex's fluxes:
+//      sum_k w_k r_k = sum_k w_k (n_x,k f_L1k + n_y,k g_L1k) + sum_k w_k (r_k - F_n(L1_k)),
+//    the first sum going into w_f, w_g (or the centre weights when L1_k is
+//    the vertex itself) and the second taken in double words.
+//    Both ends of every stencil edge are in the vertex's own stencil, so
+//    the folding adds no entries; where that fails the mesh has no precision
+//    48, and precision 64 runs in FP64 throughout, as it does where a table
+//    entry or gamma - 1 is too large or small for the double words' range.
+DivArgs div_args(fdu_mesh *m, int prec, int fin);
+fdu_status build_dw_tables(fdu_mesh *m) {
+    const int64_t ne = m->ne_act, nr = std::max<int64_t>(m->n_real, 1);
+    fdu_status st;
+    if ((st = m->alloc(m->coefdw, (size_t)kDwPairs * ne))) return st;
+    if ((st = m->alloc(m->swf48, m->vert_nnz_sell64))) return st;
+    if ((st = m->alloc(m->swg48, m->vert_nnz_sell64))) return st;
+    if ((st = m->alloc(m->swe48, m->edge_nnz_sell64))) return st;
+    if ((st = m->alloc(m->cfg48, 2 * nr))) return st;
+    int bad = 0, *dbad = m->wide;  // zero here, and again below
+    launch_coef_dw(m->coef64, m->coefdw, ne, dbad, nullptr);
+    launch_fold_tables(div_args(m, 64, 0), m->sten + 2 * ne, m->coef64 + (int64_t)kCoefN * ne,
+                       m->coef64 + (int64_t)(kCoefN + 1) * ne, m->swf48, m->swg48, m->swe48, m->cfg48, dbad, nullptr);
+    CK_LAUNCH();
+    CK(cudaMemcpy(&bad, dbad, sizeof bad, cudaMemcpyDeviceToHost));
+    CK(cudaMemset(dbad, 0, sizeof bad));
+    const double gm1 = m->opts.gamma - 1.0;
+    m->fold_ok = (bad & 1) == 0;
+    m->dw64 = bad == 0 && gm1 > 0x1p-10 && gm1 < 0x1p10;
+    return FDU_OK;
+}
+
+constexpr int kTState = 6;  // doubles of the tstate allocation
+
 // Pack host tables into device layouts.
 fdu_status upload_tables(fdu_mesh *m) {
     const HostTables &T = m->T;
@@ -314,7 +359,6 @@ fdu_status upload_tables(fdu_mesh *m) {
     Sell S32, S64;
     sell_tables(m, natural, T.wf.data(), T.wg.data(), T.we.data(), S32);
     sell_tables(m, sorted, T.wf.data(), T.wg.data(), T.we.data(), S64);
-    m->order64 = sorted;
     m->vert_nnz_sell = S32.svo[m->nslice];
     m->edge_nnz_sell = S32.seo[m->nslice];
     m->vert_nnz_sell64 = S64.svo[m->nslice];
@@ -368,10 +412,13 @@ fdu_status upload_tables(fdu_mesh *m) {
         const unsigned long long inf_bits = 0x7FF0000000000000ull;
         CK(cudaMemcpy(m->counters + 2, &inf_bits, sizeof inf_bits, cudaMemcpyHostToDevice));
     }
-    if ((st = m->alloc(m->tstate, 4))) return st;
-    CK(cudaMemset(m->tstate, 0, 4 * sizeof(double)));
+    static_assert(kWideSlots * sizeof(int) <= 2 * sizeof(double), "the wide flags share tstate's allocation");
+    if ((st = m->alloc(m->tstate, kTState))) return st;
+    CK(cudaMemset(m->tstate, 0, kTState * sizeof(double)));
+    m->nsteps = reinterpret_cast<unsigned long long *>(m->tstate + 3);
+    m->wide = reinterpret_cast<int *>(m->tstate + 4);
     CK(cudaMemset(m->wn, 0, 4 * nv * sizeof(double)));
-    return FDU_OK;
+    return build_dw_tables(m);
 }
 
 // Precision 48: the FP64 state pipeline (FP64 divergence and stage) with
@@ -379,75 +426,10 @@ fdu_status upload_tables(fdu_mesh *m) {
 inline bool fp64_state(int prec) { return prec != 32; }
 inline int prof_kind(int prec) { return prec == 64 ? 0 : prec == 32 ? 2 : 4; }
 
-// Precision 64, 32 or 48.  The first use of 48 builds its tables:
-//  - the double-word edge coefficient block (hi = the FP32 rounding of each
-//    FP64 coefficient, lo = the FP32 rounding of the remainder);
-//  - divergence tables in the FP64 SELL layout where the edge flux, which
-//    the precision-48 edge kernel leaves as the increment
-//    r_k - F_n(L1_k) = r_k - (n_x f + n_y g)(L1_k), has its left-vertex part
-//    folded into the weights of that vertex's fluxes:
-//      sum_k w_k r_k = sum_k w_k (n_x,k f_L1k + n_y,k g_L1k) + sum_k w_k (r_k - F_n(L1_k)),
-//    the first sum going into w_f, w_g (or the centre weights when L1_k is
-//    the vertex itself) and the second taken in double words.
-//    Both ends of every stencil edge are in the vertex's own stencil, so
-//    the folding adds no entries; a mesh where that fails is refused.
 fdu_status check_precision(fdu_mesh *m, int prec) {
     if (prec != 64 && prec != 32 && prec != 48) return set_err(FDU_ERR_ARG, "precision must be 64, 48 or 32");
-    if (prec != 48 || m->coefdw) return FDU_OK;
-    const HostTables &T = m->T;
-    const int64_t ne = m->ne_act, nr = m->n_real;
-    fdu_status st;
-    auto split = [](double x) {
-        const float h = (float)x;
-        return make_float2(h, (float)(x - (double)h));
-    };
-    std::vector<double> wf(T.wf), wg(T.wg), cfg(2 * std::max<int64_t>(nr, 1), 0.0);
-    for (int64_t v = 0; v < nr; ++v) {
-        const int64_t o = T.v_new2old[v];
-        double sf = 0, sg = 0, sx = 0, sy = 0;
-        for (int64_t q = T.voff[o]; q < T.voff[o + 1]; ++q) {
-            sf += T.wf[q];
-            sg += T.wg[q];
-        }
-        for (int64_t q = T.eoff[o]; q < T.eoff[o + 1]; ++q) {
-            const int32_t e = T.eid[q];
-            sx += T.we[q] * T.nrm[2 * e];
-            sy += T.we[q] * T.nrm[2 * e + 1];
-        }
-        double cf = -(sf + sx), cg = -(sg + sy);
-        for (int64_t q = T.eoff[o]; q < T.eoff[o + 1]; ++q) {
-            const int32_t e = T.eid[q];
-            const int32_t L = T.sten[6 * (int64_t)e + 2];
-            const double ax = T.we[q] * T.nrm[2 * e], ay = T.we[q] * T.nrm[2 * e + 1];
-            if (L == o) {
-                cf += ax;
-                cg += ay;
-                continue;
-            }
-            int64_t j = T.voff[o];
-            while (j < T.voff[o + 1] && T.vid[j] != L) ++j;
-            if (j == T.voff[o + 1])
-                return set_err(FDU_ERR_MESH, "precision 48: an edge's left vertex is outside the vertex's stencil");
-            wf[j] += ax;
-            wg[j] += ay;
-        }
-        cfg[v] = cf;
-        cfg[nr + v] = cg;
-    }
-    Sell S;
-    sell_tables(m, m->order64, wf.data(), wg.data(), T.we.data(), S);
-    std::vector<float2> we2(S.we.size());
-    for (size_t i = 0; i < we2.size(); ++i) we2[i] = split(S.we[i]);
-    if ((st = m->upload(m->swf48, S.wf))) return st;
-    if ((st = m->upload(m->swg48, S.wg))) return st;
-    if ((st = m->upload(m->cfg48, cfg))) return st;
-    if ((st = m->upload(m->swe48, we2))) return st;
-    float4 *k = nullptr;
-    if ((st = m->alloc(k, (size_t)kDwPairs * ne))) return st;
-    launch_coef_dw(m->coef64, k, ne, nullptr);
-    CK_LAUNCH();
-    CK(cudaDeviceSynchronize());
-    m->coefdw = k;
+    if (prec == 48 && !m->fold_ok)
+        return set_err(FDU_ERR_MESH, "precision 48: an edge's left vertex is outside the vertex's stencil");
     return FDU_OK;
 }
 
@@ -464,8 +446,9 @@ EdgeArgs edge_args(fdu_mesh *m, int prec, const void *w) {
     a.coef_gaps = !fp64_state(prec) && m->opts.f32_coef == 1;
     a.w = w;
     a.r = fp64_state(prec) ? (void *)m->r64 : (void *)m->r32;
-    if (prec == 48) {
+    if (fp64_state(prec)) {
         a.coefdw = m->coefdw;
+        a.wide = m->wide;
         dw_split(m->opts.gamma - 1.0, a.dw_gm1);
         dw_split(0.1, a.dw_tenth);
         int ee = 0;
@@ -499,11 +482,12 @@ DivArgs div_args(fdu_mesh *m, int prec, int fin) {
         a.eid = m->seid64;
         a.perm = m->perm64;
         a.wf = m->swf64; a.wg = m->swg64; a.we = m->swe64; a.cfg = m->cfg64;
-        a.F = m->F64[fin]; a.r = m->r64;
-        if (prec == 48) {  // folded vertex weights, double-word edge increments (in r64's storage)
-            a.wf = m->swf48; a.wg = m->swg48; a.we = m->swe48; a.cfg = m->cfg48;
-            a.dw_edges = true;
-        }
+        a.wf48 = m->swf48; a.wg48 = m->swg48; a.we48 = m->swe48; a.cfg48 = m->cfg48;
+        a.F = m->F64[fin]; a.r = m->r64;  // the double-word increments take r64's storage
+        a.kind = prec == 48 ? kDivDw : m->dw64 ? kDivGuard : kDivPlain;
+        a.wide = m->wide;
+        a.wide_in = fin;
+        a.wide_out = (fin + 1) % 3;
     } else {
         a.wf = m->swf32; a.wg = m->swg32; a.we = m->swe32; a.cfg = m->cfg32;
         a.F = m->F32[fin]; a.r = m->r32;
@@ -539,13 +523,26 @@ void timed(fdu_mesh *m, int kind, bool allowed, cudaStream_t s, F &&launch) {
 // Make F64[0] (or w32 and F32[0]) describe the current state wn.
 void ensure_fluxes(fdu_mesh *m, int prec, cudaStream_t s) {
     if (fp64_state(prec) && !m->f64_valid) {
-        launch_vertex_flux_f64(m->wn, m->F64[0], m->nv, m->opts.gamma, s, m->Q64[0]);
+        launch_vertex_flux_f64(m->wn, m->F64[0], m->nv, m->opts.gamma, s, m->Q64[0], m->wide, m->n_real);
         m->f64_valid = true;
     }
     if (prec == 32 && !m->f32_valid) {
         launch_vertex_flux_f32(m->wn, m->F32[0], m->w32, m->nv, m->opts.gamma, s);
         m->f32_valid = true;
     }
+}
+
+// Edge fluxes of the state whose fluxes are in buffer `in`.
+void launch_edges(fdu_mesh *m, int prec, EdgeArgs ea, int in, cudaStream_t s) {
+    if (prec == 32) {
+        launch_edge_flux_f32(ea, s);
+        return;
+    }
+    ea.Q = m->Q64[in];
+    ea.wide_in = in;
+    if (prec == 48) launch_edge_flux_dw(ea, s);
+    else if (m->dw64) launch_edge_flux_guard(ea, s);
+    else launch_edge_flux_f64(ea, s);
 }
 
 // One SSP-RK3 step: three (edge flux, divergence + stage) pairs.  Stage i
@@ -561,10 +558,7 @@ void enqueue_stages(fdu_mesh *m, int prec, double dt, const double *dt_dev, cuda
         timed(m, kd, prof, s, [&] {
             EdgeArgs ea = edge_args(m, prec, f64 ? (const void *)win : (const void *)m->w32);
             ea.dt_dev = dt_dev;
-            if (f64) ea.Q = m->Q64[stage - 1];
-            if (prec == 64) launch_edge_flux_f64(ea, s);
-            else if (prec == 48) launch_edge_flux_dw(ea, s);
-            else launch_edge_flux_f32(ea, s);
+            launch_edges(m, prec, ea, stage - 1, s);
         });
         DivArgs a = div_args(m, prec, stage - 1);
         a.wn = m->wn;
@@ -859,6 +853,7 @@ cudaError_t enqueue_step_persistent(fdu_mesh *m, int prec, cudaStream_t s, unsig
         a.Fout = f64 ? (void *)m->F64[stage % 3] : (void *)m->F32[stage % 3];
         a.Qout = f64 ? m->Q64[stage % 3] : nullptr;
         if (f64) ea.Q = m->Q64[stage - 1];
+        ea.wide_in = stage - 1;
         a.w32out = prec == 32 ? m->w32 : nullptr;
         a.comp = m->comp;
         a.dt_comp = m->dt_comp;
@@ -874,7 +869,7 @@ cudaError_t enqueue_step_persistent(fdu_mesh *m, int prec, cudaStream_t s, unsig
 // dt from there (and skip their work once t_end is reached).
 void enqueue_adaptive_step(fdu_mesh *m, int prec, double cfl, double t_end, cudaStream_t s) {
     launch_max_dt(m->wn, m->hmin, m->n_real, m->opts.gamma, m->counters + 2, s);
-    launch_dt_finalize(m->counters + 2, m->tstate, cfl, t_end, m->counters + 3, s);
+    launch_dt_finalize(m->counters + 2, m->tstate, cfl, t_end, m->nsteps, s);
     enqueue_step(m, prec, 0.0, m->tstate + 1, s, false);
 }
 
@@ -1101,8 +1096,7 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
         CK_LAUNCH();
     }
     m->f64_valid = m->f32_valid = false;
-    CK(cudaMemsetAsync(m->tstate, 0, 3 * sizeof(double), s));
-    CK(cudaMemsetAsync(m->counters + 3, 0, sizeof(unsigned long long), s));
+    CK(cudaMemsetAsync(m->tstate, 0, kTState * sizeof(double), s));
     return FDU_OK;
 }
 
@@ -1136,11 +1130,7 @@ fdu_status fdu_residual(fdu_mesh *m, int precision, double *dwdt, int on_device,
     const int kd = prof_kind(precision);
     const bool f64 = fp64_state(precision);
     timed(m, kd, true, s, [&] {
-        EdgeArgs ea = edge_args(m, precision, f64 ? (const void *)m->wn : (const void *)m->w32);
-        ea.Q = f64 ? m->Q64[0] : nullptr;
-        if (precision == 64) launch_edge_flux_f64(ea, s);
-        else if (precision == 48) launch_edge_flux_dw(ea, s);
-        else launch_edge_flux_f32(ea, s);
+        launch_edges(m, precision, edge_args(m, precision, f64 ? (const void *)m->wn : (const void *)m->w32), 0, s);
     });
     DivArgs a = div_args(m, precision, 0);
     a.out = out;
@@ -1259,7 +1249,7 @@ fdu_status fdu_advance(fdu_mesh *m, double cfl, double t_end, int precision, int
     }
     double host[3] = {0, 0, 0};
     unsigned long long n0 = 0, n1 = 0;
-    CK(cudaMemcpyAsync(&n0, m->counters + 3, sizeof n0, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(&n0, m->nsteps, sizeof n0, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(host, m->tstate, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     n1 = n0;
@@ -1271,7 +1261,7 @@ fdu_status fdu_advance(fdu_mesh *m, double cfl, double t_end, int precision, int
             for (int64_t i = 0; i < left; ++i) enqueue_adaptive_step(m, precision, cfl, t_end, s);
             CK_LAUNCH();
         }
-        CK(cudaMemcpyAsync(&n1, m->counters + 3, sizeof n1, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(&n1, m->nsteps, sizeof n1, cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(host, m->tstate, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (host[1] == 0.0 && host[0] < t_end && host[2] == 0.0) break;  // no progress
@@ -1377,7 +1367,7 @@ fdu_status fdu_batch_create(int32_t n_meshes, const double *const *xy, const int
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
         m->pl_threads = 256;
-        m->pl_blocks = sms * std::max(1, persistent_blocks_per_sm(32, 256));
+        m->pl_blocks = sms * std::max(1, persistent_blocks_per_sm(32, 256, false));
         if (cudaGetLastError() != cudaSuccess) st = set_err(FDU_ERR_CUDA, "batch setup");
     }
     if (st != FDU_OK) {
@@ -1443,7 +1433,7 @@ fdu_status fdu_batch_set_launch(fdu_mesh *m, int threads, int blocks_per_sm) {
     if (threads != 128 && threads != 256 && threads != 512) return set_err(FDU_ERR_ARG, "threads must be 128, 256, 512");
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-    const int occ = std::max(persistent_blocks_per_sm(64, threads), persistent_blocks_per_sm(32, threads));
+    const int occ = std::max(persistent_blocks_per_sm(64, threads, m->dw64), persistent_blocks_per_sm(32, threads, false));
     if (blocks_per_sm < 1 || blocks_per_sm > occ)
         return set_err(FDU_ERR_ARG, "blocks_per_sm must be 1.." + std::to_string(occ) + " at " +
                                         std::to_string(threads) + " threads");
@@ -1474,7 +1464,7 @@ fdu_status fdu_batch_rk_steps(fdu_mesh *m, int precision, int n_steps, void *str
     if ((st = check_precision(m, precision))) return st;
     if (n_steps == 0) return FDU_OK;
     cudaStream_t s = m->stream(stream);
-    const int occ = persistent_blocks_per_sm(precision, m->pl_threads);
+    const int occ = persistent_blocks_per_sm(precision, m->pl_threads, m->dw64);
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
     if (occ < 1) return set_err(FDU_ERR_ARG, "the persistent kernel does not fit " + std::to_string(m->pl_threads) +
@@ -1524,7 +1514,7 @@ fdu_status fdu_batch_autotune(fdu_mesh *m, int precision, int *threads, int *blo
     double best = INFINITY;
     int bt = m->pl_threads, bb = m->pl_blocks / std::max(sms, 1);
     for (int t : {128, 256, 512}) {
-        const int occ = persistent_blocks_per_sm(precision, t);
+        const int occ = persistent_blocks_per_sm(precision, t, m->dw64);
         for (int k = 1; k <= occ; ++k) {
             m->pl_threads = t;
             m->pl_blocks = k * sms;
@@ -1583,7 +1573,7 @@ fdu_status fdu_batch_barrier_selftest(fdu_mesh *m, int *status) {
     a.dt_comp = m->dt_comp;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-    const int nb = std::min(m->pl_blocks, persistent_blocks_per_sm(32, m->pl_threads) * sms);
+    const int nb = std::min(m->pl_blocks, persistent_blocks_per_sm(32, m->pl_threads, false) * sms);
     CK(launch_stage_persistent(32, 1, ea, a, m->bar, m->bar + 1, (unsigned)nb + 1, 20000, m->bar_err, m->pl_threads,
                                nb, s));
     // an ordinary step enqueued behind the failed launch, before the error is
@@ -1625,8 +1615,11 @@ fdu_status fdu_residual_noalloc(const fdu_mesh *mc, const double *w, double *dwd
     launch_vertex_flux_f64(wi, F, m->nv, m->opts.gamma, s);
     EdgeArgs ea = edge_args(m, 64, wi);
     ea.r = r;
+    ea.wide = nullptr;
     launch_edge_flux_f64(ea, s);
     DivArgs a = div_args(m, 64, 0);
+    a.kind = kDivPlain;
+    a.wide = nullptr;
     a.F = F;
     a.r = r;
     a.out = dwdt;

@@ -60,17 +60,20 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) edge_flux_dw_kernel(EdgeArgs A)
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= A.ne) return;
     if (A.dt_dev && *A.dt_dev == 0.0) return;
-    edge_flux_dw_body(A, e, Stage{stage + threadIdx.x, kEdgeBlock});
+    clear_wide(A, e);
+    edge_flux_dw_body<false>(A, e, Stage{stage + threadIdx.x, kEdgeBlock});
 }
 
 // The edge coefficient block as paired double words: hi = the FP32 rounding
 // of a value, lo = the FP32 rounding of the remainder.
-__global__ void coef_dw_kernel(const double *__restrict__ coef, float4 *__restrict__ out, int64_t ne) {
+__global__ void coef_dw_kernel(const double *__restrict__ coef, float4 *__restrict__ out, int64_t ne,
+                               int *bad) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= ne) return;
 #pragma unroll
     for (int p = 0; p < kDwPairs; ++p) {
         const double a = coef[(int64_t)dw_pair(p, 0) * ne + e], b = coef[(int64_t)dw_pair(p, 1) * ne + e];
+        if (!(fabs(a) < kDwMax && fabs(b) < kDwMax)) atomicOr(bad, 2);
         const float ah = __double2float_rn(a), bh = __double2float_rn(b);
         out[(int64_t)p * ne + e] = make_float4(ah, bh, __double2float_rn(a - (double)ah), __double2float_rn(b - (double)bh));
     }
@@ -108,8 +111,8 @@ void launch_dw_check(int op, const double *x, const double *y, double *z, int64_
     if (n > 0) dw_check_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(op, x, y, z, n);
 }
 
-void launch_coef_dw(const double *coef, float4 *coefdw, int64_t ne, cudaStream_t s) {
-    if (ne > 0) coef_dw_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(coef, coefdw, ne);
+void launch_coef_dw(const double *coef, float4 *coefdw, int64_t ne, int *bad, cudaStream_t s) {
+    if (ne > 0) coef_dw_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(coef, coefdw, ne, bad);
 }
 
 void launch_edge_flux_dw(const EdgeArgs &a, cudaStream_t s) {

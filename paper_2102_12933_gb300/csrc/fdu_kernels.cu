@@ -31,7 +31,7 @@ namespace {
 using namespace dev;
 
 // ------------------------------------------------------------------ FP64 edge flux
-__device__ __forceinline__ void edge_flux_f64_body(const EdgeArgs &A, const int64_t e) {
+__device__ __forceinline__ dbl4 edge_flux_f64_value(const EdgeArgs &A, const int64_t e) {
     const double *__restrict__ w = static_cast<const double *>(A.w);
     const double *__restrict__ coef = static_cast<const double *>(A.coef);
     const double gm1 = A.gm1, hgm1 = A.hgm1;
@@ -111,7 +111,48 @@ __device__ __forceinline__ void edge_flux_f64_body(const EdgeArgs &A, const int6
     f.y = fma(wl.y, qnl, fma(pl.p, nx, D.y));
     f.z = fma(wl.z, qnl, fma(pl.p, ny, D.z));
     f.w = fma(wl.w + pl.p, qnl, D.w);
-    st4(static_cast<double *>(A.r), e, f);
+    return f;
+}
+__device__ __forceinline__ void edge_flux_f64_body(const EdgeArgs &A, const int64_t e) {
+    st4(static_cast<double *>(A.r), e, edge_flux_f64_value(A, e));
+}
+// Precision 64 off the double-word path, out of line so that its registers do
+// not weigh on that path: the flux r in FP64 (a stage that runs in FP64
+// throughout), or its increment r - F_n(L1) as the double words the folded
+// divergence reads (a single edge).
+__device__ __noinline__ void edge_flux_f64_cold(const EdgeArgs *A, const int64_t e, const bool increment) {
+    dbl4 f = edge_flux_f64_value(*A, e);
+    if (increment) {
+        const dbl4 L1 = ld4v(static_cast<const double *>(A->w), __ldg(A->sten + 2 * A->ne + e));
+        const double *coef = static_cast<const double *>(A->coef);
+        const double nx = __ldg(coef + (int64_t)kCoefN * A->ne + e), ny = __ldg(coef + (int64_t)(kCoefN + 1) * A->ne + e);
+        const Prim64 P = prim64(L1, A->gm1);
+        const double mn = fma(L1.y, nx, L1.z * ny), q = mn * P.ir;
+        using namespace dwa;
+        const dw x = d2dw(f.x - mn), y = d2dw(f.y - fma(L1.y, q, P.p * nx)), z = d2dw(f.z - fma(L1.z, q, P.p * ny)),
+                 w = d2dw(f.w - (L1.w + P.p) * q);
+        float4 *r = static_cast<float4 *>(A->r);
+        r[2 * e] = make_float4(x.h, x.l, y.h, y.l);
+        r[2 * e + 1] = make_float4(z.h, z.l, w.h, w.l);
+        return;
+    }
+    st4(static_cast<double *>(A->r), e, f);
+}
+// One edge at precision 64.
+__device__ __forceinline__ void edge_flux_guard_body(const EdgeArgs &A, const int64_t e, const dwa::Stage &S,
+                                                     const bool wide) {
+    if (wide) edge_flux_f64_cold(&A, e, false);
+    else if (!dwa::edge_flux_dw_body<true>(A, e, S)) edge_flux_f64_cold(&A, e, true);
+}
+__device__ __forceinline__ bool stage_is_wide(const int *wide, int in) {
+    return (__ldcg(wide + in) | __ldcg(wide + kWideGhost)) != 0;
+}
+// A state outside the double words' window: density or energy not in
+// [2^-kWideExp, 2^kWideExp), by the exponent field (NaN, zero, negative and
+// infinite values fail).
+__device__ __forceinline__ bool outside_window(const dbl4 &w) {
+    const unsigned lo = (unsigned)(1023 - kWideExp) << 20, n = (unsigned)(2 * kWideExp) << 20;
+    return (unsigned)__double2hiint(w.x) - lo >= n || (unsigned)__double2hiint(w.w) - lo >= n;
 }
 
 // ------------------------------------------------------------------ vertex fluxes
@@ -129,7 +170,7 @@ __device__ __forceinline__ dbl4 roe_record64(const dbl4 &w, const Prim64 &P) {
 }
 
 __global__ void vertex_flux_f64_kernel(const double *__restrict__ w, double *__restrict__ F, double *__restrict__ Q,
-                                       int64_t n, double gm1) {
+                                       int64_t n, double gm1, int *wide, int64_t n_real) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
     const dbl4 s = ld4(w, v);
@@ -139,6 +180,7 @@ __global__ void vertex_flux_f64_kernel(const double *__restrict__ w, double *__r
     st4(F, 2 * v, f);
     st4(F, 2 * v + 1, g);
     if (Q) st4(Q, v, roe_record64(s, P));
+    if (wide && outside_window(s)) wide[v < n_real ? 0 : kWideGhost] = 1;
 }
 
 // Forward-Euler part of an SSP-RK3 stage, fe = ws + theta dt L.  Without
@@ -217,8 +259,8 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
     const int64_t v = A.perm ? (int64_t)__ldg(A.perm + i) : i;
     const double *__restrict__ F = static_cast<const double *>(A.F);
     const double *__restrict__ r = static_cast<const double *>(A.r);
-    const double *__restrict__ wf = static_cast<const double *>(A.wf);
-    const double *__restrict__ wg = static_cast<const double *>(A.wg);
+    const double *__restrict__ wf = DWE ? A.wf48 : static_cast<const double *>(A.wf);
+    const double *__restrict__ wg = DWE ? A.wg48 : static_cast<const double *>(A.wg);
     const double *__restrict__ we = static_cast<const double *>(A.we);
     dbl4 acc = dbl4_make(0, 0, 0, 0);
     {
@@ -236,7 +278,7 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
     }
     if (DWE) {
         using namespace dwa;
-        const float2 *__restrict__ we2 = static_cast<const float2 *>(A.we);
+        const float2 *__restrict__ we2 = A.we48;
         const float4 *__restrict__ rd = static_cast<const float4 *>(A.r);
         dot2 sx{0.0f, 0.0f}, sy = sx, sz = sx, sw = sx;
         const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = __ldg(A.slice_eoff + sl + 1);
@@ -271,7 +313,7 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
         }
     }
     {
-        const double *cfg = static_cast<const double *>(A.cfg);
+        const double *cfg = DWE ? A.cfg48 : static_cast<const double *>(A.cfg);
         const double cf = __ldg(cfg + v), cg = __ldg(cfg + A.n_real + v);
         const dbl4 f = ld4v(F, 2 * v), g = ld4v(F, 2 * v + 1);
         acc.x = fma(cf, f.x, fma(cg, g.x, acc.x));
@@ -308,6 +350,17 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
     st4(Fo, 2 * v, f);
     st4(Fo, 2 * v + 1, g);
     if (A.Qout) st4(A.Qout, v, roe_record64(o, P));
+    if (A.wide && outside_window(o)) A.wide[A.wide_out] = 1;
+}
+// The FP64 form out of line, for the kernels that seldom take it.
+template <int MODE>
+__device__ __noinline__ void div_f64_cold(const DivArgs *A, const int64_t i) { div_f64_body<MODE, false>(*A, i); }
+// The divergence of one vertex by KIND (kDivPlain, kDivDw, kDivGuard).
+template <int MODE, int KIND>
+__device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, const bool wide) {
+    if (KIND == kDivPlain) div_f64_body<MODE, false>(A, i);
+    else if (KIND == kDivGuard && wide) div_f64_cold<MODE>(&A, i);
+    else div_f64_body<MODE, true>(A, i);
 }
 
 // ================================================================== FP32 path
@@ -712,12 +765,80 @@ __global__ void __launch_bounds__(kEdgeBlock, GAPS ? 6 : 5) edge_flux_f32_kernel
     if (A.dt_dev && *A.dt_dev == 0.0) return;  // adaptive run already at t_end
     edge_flux_f32_body<GAPS>(A, e);
 }
-template <int MODE, bool DWE>
-__global__ void __launch_bounds__(kDivBlock) div_f64_kernel(DivArgs A) {
+// Precision 64: the double-word edge flux, or FP64 where the state is outside
+// its window or an edge fails its guard (edge_flux_dw_body).  In FP64 throughout
+// the kernel is bound by GB300's FP64 pipe (449 instructions per edge, each 64
+// cycles of a sub-partition's pipe, 90 % busy): 0.618 ms at 250k vertices, and
+// the divergence after it 0.186 ms; on the double-word path 0.119 and 0.128 ms.
+// Error of the residual against plain FP64 (vortex 40^2 / Riemann 101^2 / Sod
+// 55^2 of degree 5): 2.3e-14 / 6.5e-14 / 2.2e-14 before, 6.9e-15 / 3.4e-15 /
+// 1.1e-14 now: the increments are small against the state, and the folded
+// weights leave fewer large terms to cancel in the divergence.
+__global__ void __launch_bounds__(kEdgeBlock, 4) edge_flux_guard_kernel(const __grid_constant__ EdgeArgs A) {
+    __shared__ float4 stage[dwa::kDwSlots * kEdgeBlock];
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= A.ne) return;
+    if (A.dt_dev && *A.dt_dev == 0.0) return;
+    dwa::clear_wide(A, e);
+    edge_flux_guard_body(A, e, dwa::Stage{stage + threadIdx.x, kEdgeBlock}, stage_is_wide(A.wide, A.wide_in));
+}
+template <int MODE, int KIND>
+__global__ void __launch_bounds__(kDivBlock) div_f64_kernel(const __grid_constant__ DivArgs A) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= A.n_real) return;
     if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;  // adaptive run already at t_end
-    div_f64_body<MODE, DWE>(A, v);
+    div_f64_any<MODE, KIND>(A, v, KIND == kDivGuard && stage_is_wide(A.wide, A.wide_in));
+}
+// Folded tables of the double-word divergence (launch_fold_tables); thread i
+// serves SELL position i.  Entries and sums in the order of the SELL lists,
+// rounded one by one.
+__global__ void fold_tables_kernel(DivArgs A, const int32_t *__restrict__ left, const double *__restrict__ nx,
+                                   const double *__restrict__ ny, double *wf48, double *wg48, float2 *we48,
+                                   double *cfg48, int *bad) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t sl = i / kSell;
+    if (sl >= (A.n_real + kSell - 1) / kSell) return;
+    const int lane = (int)(i % kSell);
+    const int64_t vb = A.slice_voff[sl] + lane, ve = A.slice_voff[sl + 1];
+    const int64_t eb = A.slice_eoff[sl] + lane, ee = A.slice_eoff[sl + 1];
+    const double *wf = static_cast<const double *>(A.wf), *wg = static_cast<const double *>(A.wg);
+    const double *we = static_cast<const double *>(A.we), *cfg = static_cast<const double *>(A.cfg);
+    int flag = 0;
+    for (int64_t p = vb; p < ve; p += kSell) {
+        wf48[p] = wf[p];
+        wg48[p] = wg[p];
+        if (!(fabs(wf[p]) < kDwMax && fabs(wg[p]) < kDwMax)) flag |= 2;
+    }
+    const bool real = i < A.n_real;
+    const int32_t v = real ? A.perm[i] : 0;
+    double cf = real ? cfg[v] : 0.0, cg = real ? cfg[A.n_real + v] : 0.0;
+    for (int64_t q = eb; q < ee; q += kSell) {
+        const double w = we[q];
+        const float h = __double2float_rn(w);
+        we48[q] = make_float2(h, __double2float_rn(w - (double)h));
+        if (!(fabs(w) < kDwMax)) flag |= 2;
+        if (w == 0.0) continue;  // padding
+        const int32_t e = A.eid[q], L = left[e];
+        const double ax = __dmul_rn(w, nx[e]), ay = __dmul_rn(w, ny[e]);
+        if (L == v) {
+            cf = __dadd_rn(cf, ax);
+            cg = __dadd_rn(cg, ay);
+            continue;
+        }
+        int64_t p = vb;
+        while (p < ve && A.vid[p] != L) p += kSell;
+        if (p >= ve) {
+            flag |= 1;
+            continue;
+        }
+        wf48[p] = __dadd_rn(wf48[p], ax);
+        wg48[p] = __dadd_rn(wg48[p], ay);
+    }
+    if (real) {
+        cfg48[v] = cf;
+        cfg48[A.n_real + v] = cg;
+    }
+    if (flag) atomicOr(bad, flag);
 }
 template <int MODE>
 __global__ void __launch_bounds__(kDivBlock) div_f32_kernel(DivArgs A) {
@@ -801,22 +922,28 @@ __global__ void stage_persistent_kernel(EdgeArgs EA, DivArgs DA, unsigned int *b
     }
 }
 
-// Precision 48: the same stage with the double-word edge flux (its staging in
+// Precision 48, and with GUARD precision 64: the same stage with the double-word edge flux (its staging in
 // dynamic shared memory, kDwSlots 16-byte slots per thread) and the folded
 // divergence.  At most 512 threads a block, so at most 128 registers.
-template <int MODE>
+template <int MODE, bool GUARD>
 __global__ void __launch_bounds__(512, 1)
-    stage_persistent_dw_kernel(EdgeArgs EA, DivArgs DA, unsigned int *bar_count, unsigned int *bar_gen,
-                               unsigned int nblocks_expected, unsigned long long spin_limit, int *err) {
+    stage_persistent_dw_kernel(const __grid_constant__ EdgeArgs EA, const __grid_constant__ DivArgs DA,
+                               unsigned int *bar_count, unsigned int *bar_gen, unsigned int nblocks_expected,
+                               unsigned long long spin_limit, int *err) {
     if (barrier_failed(err)) return;
     extern __shared__ float4 dw_stage[];
     const dwa::Stage T{dw_stage + threadIdx.x, (int)blockDim.x};
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t e = t0; e < EA.ne; e += stride) dwa::edge_flux_dw_body(EA, e, T);
+    const bool wide = GUARD && stage_is_wide(EA.wide, EA.wide_in);
+    for (int64_t e = t0; e < EA.ne; e += stride) {
+        dwa::clear_wide(EA, e);
+        if (GUARD) edge_flux_guard_body(EA, e, T, wide);
+        else dwa::edge_flux_dw_body<false>(EA, e, T);
+    }
     __threadfence();
     if (!grid_barrier(bar_count, bar_gen, nblocks_expected, spin_limit, err)) return;
-    for (int64_t v = t0; v < DA.n_real; v += stride) div_f64_body<MODE, true>(DA, v);
+    for (int64_t v = t0; v < DA.n_real; v += stride) div_f64_any<MODE, GUARD ? kDivGuard : kDivDw>(DA, v, wide);
 }
 
 // ------------------------------------------------------------------ support kernels
@@ -942,8 +1069,15 @@ inline unsigned blocks(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 }  // namespace
 
-void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q) {
-    if (n > 0) vertex_flux_f64_kernel<<<blocks(n, 256), 256, 0, s>>>(w, F, Q, n, gamma - 1.0);
+void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q, int *wide,
+                            int64_t n_real) {
+    if (n > 0) vertex_flux_f64_kernel<<<blocks(n, 256), 256, 0, s>>>(w, F, Q, n, gamma - 1.0, wide, n_real);
+}
+void launch_fold_tables(const DivArgs &a, const int32_t *left, const double *nx, const double *ny, double *wf48,
+                        double *wg48, float2 *we48, double *cfg48, int *bad, cudaStream_t s) {
+    if (a.n_real <= 0) return;
+    const int64_t n = (a.n_real + kSell - 1) / kSell * kSell;
+    fold_tables_kernel<<<blocks(n, 128), 128, 0, s>>>(a, left, nx, ny, wf48, wg48, we48, cfg48, bad);
 }
 void launch_vertex_flux_f32(const double *w, float4 *F, float4 *w32, int64_t n, double gamma, cudaStream_t s) {
     if (n > 0) vertex_flux_f32_kernel<<<blocks(n, 256), 256, 0, s>>>(w, F, w32, n, (float)(gamma - 1.0));
@@ -951,25 +1085,29 @@ void launch_vertex_flux_f32(const double *w, float4 *F, float4 *w32, int64_t n, 
 void launch_edge_flux_f64(const EdgeArgs &a, cudaStream_t s) {
     if (a.ne > 0) edge_flux_f64_kernel<<<blocks(a.ne, kEdgeBlock), kEdgeBlock, 0, s>>>(a);
 }
+void launch_edge_flux_guard(const EdgeArgs &a, cudaStream_t s) {
+    if (a.ne > 0) edge_flux_guard_kernel<<<blocks(a.ne, kEdgeBlock), kEdgeBlock, 0, s>>>(a);
+}
 void launch_edge_flux_f32(const EdgeArgs &a, cudaStream_t s) {
     if (a.ne <= 0) return;
     if (a.coef_gaps) edge_flux_f32_kernel<true><<<blocks(a.ne, kEdgeBlock), kEdgeBlock, 0, s>>>(a);
     else edge_flux_f32_kernel<false><<<blocks(a.ne, kEdgeBlock), kEdgeBlock, 0, s>>>(a);
 }
-template <bool DWE>
+template <int KIND>
 void launch_div_f64_t(const DivArgs &a, int mode, cudaStream_t s) {
     const unsigned g = blocks(a.n_real, kDivBlock);
     switch (mode) {
-        case 0: div_f64_kernel<0, DWE><<<g, kDivBlock, 0, s>>>(a); break;
-        case 1: div_f64_kernel<1, DWE><<<g, kDivBlock, 0, s>>>(a); break;
-        case 2: div_f64_kernel<2, DWE><<<g, kDivBlock, 0, s>>>(a); break;
-        default: div_f64_kernel<3, DWE><<<g, kDivBlock, 0, s>>>(a); break;
+        case 0: div_f64_kernel<0, KIND><<<g, kDivBlock, 0, s>>>(a); break;
+        case 1: div_f64_kernel<1, KIND><<<g, kDivBlock, 0, s>>>(a); break;
+        case 2: div_f64_kernel<2, KIND><<<g, kDivBlock, 0, s>>>(a); break;
+        default: div_f64_kernel<3, KIND><<<g, kDivBlock, 0, s>>>(a); break;
     }
 }
 void launch_div_f64(const DivArgs &a, int mode, cudaStream_t s) {
     if (a.n_real <= 0) return;
-    if (a.dw_edges) launch_div_f64_t<true>(a, mode, s);
-    else launch_div_f64_t<false>(a, mode, s);
+    if (a.kind == kDivGuard) launch_div_f64_t<kDivGuard>(a, mode, s);
+    else if (a.kind == kDivDw) launch_div_f64_t<kDivDw>(a, mode, s);
+    else launch_div_f64_t<kDivPlain>(a, mode, s);
 }
 void launch_div_f32(const DivArgs &a, int mode, cudaStream_t s) {
     if (a.n_real <= 0) return;
@@ -1013,17 +1151,17 @@ cudaError_t coop(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigne
 
 namespace {
 size_t dw_stage_bytes(int threads) { return (size_t)dwa::kDwSlots * sizeof(float4) * threads; }
-template <int MODE>
+template <int MODE, bool GUARD>
 cudaError_t coop48(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigned int *g, unsigned int ne,
                    unsigned long long lim, int *err, int threads, int nb, cudaStream_t s) {
     EdgeArgs a = ea;
     DivArgs d = da;
     void *args[] = {&a, &d, &c, &g, &ne, &lim, &err};
     const size_t bytes = dw_stage_bytes(threads);
-    cudaError_t e = cudaFuncSetAttribute((const void *)stage_persistent_dw_kernel<MODE>,
+    cudaError_t e = cudaFuncSetAttribute((const void *)stage_persistent_dw_kernel<MODE, GUARD>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
-    return cudaLaunchCooperativeKernel((const void *)stage_persistent_dw_kernel<MODE>, dim3(nb), dim3(threads), args,
+    return cudaLaunchCooperativeKernel((const void *)stage_persistent_dw_kernel<MODE, GUARD>, dim3(nb), dim3(threads), args,
                                        bytes, s);
 }
 }  // namespace
@@ -1033,9 +1171,14 @@ cudaError_t launch_stage_persistent(int prec, int mode, const EdgeArgs &ea, cons
                                     unsigned long long spin_limit, int *err, int threads, int nb, cudaStream_t s) {
     const unsigned int ne = nblocks_expected;
     if (prec == 48) {
-        if (mode == 1) return coop48<1>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
-        if (mode == 2) return coop48<2>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
-        return coop48<3>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+        if (mode == 1) return coop48<1, false>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+        if (mode == 2) return coop48<2, false>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+        return coop48<3, false>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+    }
+    if (prec == 64 && da.kind == kDivGuard) {
+        if (mode == 1) return coop48<1, true>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+        if (mode == 2) return coop48<2, true>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+        return coop48<3, true>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
     }
     if (prec == 64) {
         if (mode == 1) return coop<64, 1>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
@@ -1047,20 +1190,30 @@ cudaError_t launch_stage_persistent(int prec, int mode, const EdgeArgs &ea, cons
     return coop<32, 3>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
 }
 
-int persistent_blocks_per_sm(int prec, int threads) {
+namespace {
+template <bool GUARD>
+int dw_blocks_per_sm(int threads) {
+    int n = 0;
+    const size_t bytes = dw_stage_bytes(threads);
+    for (auto k : {stage_persistent_dw_kernel<1, GUARD>, stage_persistent_dw_kernel<2, GUARD>,
+                   stage_persistent_dw_kernel<3, GUARD>})
+        if (cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+            return 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_dw_kernel<3, GUARD>, threads, bytes);
+    return n;
+}
+}  // namespace
+
+int persistent_blocks_per_sm(int prec, int threads, bool guard) {
     int n = 0;
     // the three stage modes share their register footprint; mode 3 stands for all
-    if (prec == 48) {
-        const size_t bytes = dw_stage_bytes(threads);
-        for (auto k : {stage_persistent_dw_kernel<1>, stage_persistent_dw_kernel<2>, stage_persistent_dw_kernel<3>})
-            if (cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
-                cudaSuccess)
-                return 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_dw_kernel<3>, threads, bytes);
-    } else if (prec == 64)
+    if (prec == 48) return dw_blocks_per_sm<false>(threads);
+    if (prec == 64) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<64, 3>, threads, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<32, 3>, threads, 0);
+        // a block the FP64 kernel has no registers for is refused at precision 64 on either path
+        return guard && n > 0 ? dw_blocks_per_sm<true>(threads) : n;
+    }
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<32, 3>, threads, 0);
     return n;
 }
 

@@ -10,6 +10,20 @@ constexpr int kSell = 32;        // SELL slice width of the divergence tables (o
 constexpr int kEdgeBlock = 128;  // threads per block, edge-flux kernels
 constexpr int kDivBlock = 128;   // threads per block, divergence kernels
 
+// Precision 64 takes an edge's increments in double words where FP32's exponent
+// range holds them.  The kernels that write a state's fluxes (vertex_flux, the
+// stage epilogues) check every vertex: density and energy within 2^+-kWideExp,
+// so that squares and products of the edge flux stay far from 2^+-126.  wide[i]
+// is non-zero when the state of flux buffer i (0..2) failed, wide[3] when a
+// ghost of the state that was set did (Dirichlet ghosts keep it).  A stage
+// that finds wide[in] or wide[3] set runs in FP64 throughout; the edge kernel
+// of each stage clears the slot that the stage after it writes (the buffers
+// rotate, and nothing reads that slot in between).
+constexpr int kWideGhost = 3;
+constexpr int kWideSlots = 4;
+constexpr int kWideExp = 24;
+constexpr double kDwMax = 0x1p40;  // largest table entry of the double-word path of precision 64
+
 // Edge-flux inputs (internal ids, SoA over the active edges).
 struct EdgeArgs {
     const int32_t *sten;  // [6][ne]  L3 L2 L1 R1 R2 R3
@@ -33,7 +47,17 @@ struct EdgeArgs {
     float dw_tenth[2];    // 0.1 as a double word
     float dw_eps[2];      // WENO epsilon = dw_eps * 2^dw_eps_e, dw_eps in [1, 2)
     int dw_eps_e;
+    // precision 64 and 48: whether a state left the double words' window
+    // (WideFlags), and the buffer slot of the stage state; nullptr: FP64 only
+    int *wide;
+    int wide_in;
 };
+
+
+// Divergence of an FP64 state: plain FP64 tables and edge fluxes; double-word
+// edge increments with the folded tables (precision 48); or by the wide flags
+// either of the two (precision 64).
+enum { kDivPlain = 0, kDivDw = 1, kDivGuard = 2 };
 
 // Divergence (+ optional SSP-RK3 stage) inputs.
 struct DivArgs {
@@ -43,12 +67,18 @@ struct DivArgs {
     const int32_t *perm;         // [n_real] vertex at each SELL position (nullptr = position i is vertex i)
     const int32_t *vid;          // vertex entries (SELL: entry j of lane l at off + 32 j + l)
     const void *wf, *wg;         // weights of f_j and g_j
+    // precision 64 and 48: folded vertex weights, double-word edge weights and
+    // centre weights that go with the double-word edge increments
+    const double *wf48, *wg48, *cfg48;
+    const float2 *we48;
     const int32_t *eid;          // edge entries
-    const void *we;              // weights of r_k (double words when dw_edges)
+    const void *we;              // weights of r_k
     const void *cfg;             // [2][n_real] centre weights: -(sum wf + sum we nx), -(sum wg + sum we ny)
     const void *F;               // vertex fluxes of the stage state: FP64 [nv][8] (f0..3, g0..3); FP32 [nv][2] float4 pairs
-    const void *r;               // edge fluxes (dw_edges: the precision-48 edge increments)
-    bool dw_edges;               // precision 48: folded vertex weights, double-word edge part
+    const void *r;               // edge fluxes (double-word edge increments for kDivDw)
+    int kind;                    // FP64 state: kDivPlain, kDivDw or kDivGuard
+    int *wide;                   // WideFlags (nullptr: not kept), and the slots of the stage's input and output
+    int wide_in, wide_out;
     // residual output (mode 0)
     double *out;                 // [nv][4] FP64
     const int32_t *out_map;      // internal -> output row (nullptr = internal order)
@@ -70,13 +100,22 @@ struct DivArgs {
 };
 
 // F[v] = (f, g) of w[v]; Q (optional) = Roe records (sqrt rho, sqrt rho u, sqrt rho v, sqrt rho H)
-void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q = nullptr);
+// wide (optional): slot 0 of the WideFlags for vertices below n_real, kWideGhost for the others
+void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q = nullptr,
+                            int *wide = nullptr, int64_t n_real = 0);
 void launch_vertex_flux_f32(const double *w, float4 *F, float4 *w32, int64_t n, double gamma, cudaStream_t s);
-void launch_edge_flux_f64(const EdgeArgs &a, cudaStream_t s);
+void launch_edge_flux_f64(const EdgeArgs &a, cudaStream_t s);    // FP64 throughout
+void launch_edge_flux_guard(const EdgeArgs &a, cudaStream_t s);  // precision 64: double words within the window
 void launch_edge_flux_f32(const EdgeArgs &a, cudaStream_t s);
 void launch_edge_flux_dw(const EdgeArgs &a, cudaStream_t s);
+// Folded divergence tables from the FP64 SELL tables in `a` (n_real, perm,
+// slices, ids, wf, wg, we, cfg), the edges' left vertices and normals; *bad |= 1
+// where an edge's left vertex is outside a vertex's stencil, |= 2 where a
+// weight or coefficient is beyond the double words' window.
+void launch_fold_tables(const DivArgs &a, const int32_t *left, const double *nx, const double *ny, double *wf48,
+                        double *wg48, float2 *we48, double *cfg48, int *bad, cudaStream_t s);
 // coefdw[kDwPairs][ne] = the double words of coef[kEdgeCoef][ne], paired
-void launch_coef_dw(const double *coef, float4 *coefdw, int64_t ne, cudaStream_t s);
+void launch_coef_dw(const double *coef, float4 *coefdw, int64_t ne, int *bad, cudaStream_t s);
 // z = double-word primitive `op` of x (and y), device pointers (accuracy check)
 void launch_dw_check(int op, const double *x, const double *y, double *z, int64_t n, cudaStream_t s);
 void launch_div_f64(const DivArgs &a, int mode, cudaStream_t s);
@@ -110,7 +149,8 @@ void launch_max_dt(const double *w, const double *hmin, int64_t n, double gamma,
 cudaError_t launch_stage_persistent(int prec, int mode, const EdgeArgs &ea, const DivArgs &da, unsigned int *bar_count,
                                     unsigned int *bar_gen, unsigned int nblocks_expected,
                                     unsigned long long spin_limit, int *err, int threads, int blocks, cudaStream_t s);
-// Co-resident blocks per SM of the persistent stage kernel at `threads`.
-int persistent_blocks_per_sm(int prec, int threads);
+// Co-resident blocks per SM of the persistent stage kernel at `threads`; guard:
+// the mesh's precision-64 kernel takes the double-word path (kDivGuard).
+int persistent_blocks_per_sm(int prec, int threads, bool guard);
 
 }  // namespace fdu

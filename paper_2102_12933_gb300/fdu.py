@@ -360,9 +360,10 @@ class Mesh:
     def residual(self, precision=64, out=None, stream=None):
         """dw/dt of the current state, [nv, 4] in the caller's vertex order
         (edge fluxes by characteristic NU-WENO5 and a Roe flux, Section 2.3.1;
-        least-squares divergence, Section 2.2.1).  precision 64: FP64;
-        48: the FP64 result with the edge-flux increments in double-word FP32;
-        32: FP32 fluxes with FP64 accumulation.  out: a host array or a CUDA
+        least-squares divergence, Section 2.2.1).  precision 64: FP64 accuracy
+        (state-sized terms FP64, edge-flux increments double-word FP32 within
+        its range, FP64 outside it); 48: the double-word form without the range
+        checks; 32: FP32 fluxes with FP64 accumulation.  out: a host array or a CUDA
         tensor of that shape (None: a new host array)."""
         if out is None:
             out = np.zeros((self.nv, 4))
