@@ -67,6 +67,7 @@ struct fdu_mesh {
     float4 *coefdw = nullptr;
     double *swf48 = nullptr, *swg48 = nullptr, *cfg48 = nullptr;
     float2 *swe48 = nullptr;
+    TileTables tile32{};              // FP32 divergence tiles (smem = 0: not used)
     bool fold_ok = false;             // the folded tables hold (precision 48 is available)
     bool dw64 = false;                // precision 64 takes the double-word path (fold_ok, tables in its window)
     int64_t *slice_voff = nullptr, *slice_eoff = nullptr;       // FP32 layout (natural order)
@@ -260,6 +261,68 @@ void stencil_gaps(const double xi[6], float g[4]) {
 //    the folding adds no entries; where that fails the mesh has no precision
 //    48, and precision 64 runs in FP64 throughout, as it does where a table
 //    entry or gamma - 1 is too large or small for the double words' range.
+// FP32 divergence tiles, formed on the device from the FP32 SELL tables: sizes
+// first (read back to place the lists), then lists, positions and weights.
+// T.smem stays 0, and the divergence gathers from global memory, where a tile
+// has too many distinct vertices or edges: a vertex order without locality
+// (renumber = 0 on shuffled ids), whose staging would copy more than it saves.
+fdu_status build_tiles(fdu_mesh *m) {
+    constexpr int kSlices = kTile / kSell;
+    constexpr int kMaxBytes = 48 * 1024;  // shared memory of a launch without opt-in
+    TileTables T{};
+    T.ntiles = (m->n_real + kTile - 1) / kTile;
+    const int64_t nt = T.ntiles, ns = nt * kSlices;
+    if (nt == 0) return FDU_OK;
+    const TileSource S{m->n_real, m->slice_voff, m->slice_eoff, m->svid, m->seid, m->swf32, m->swg32, m->swe32};
+    // one allocation: the positions' order, the offsets (nt + 1, nt + 1, ns + 1, ns + 1)
+    const int64_t noff = 2 * (nt + 1) + 2 * (ns + 1);
+    int32_t *base = nullptr;
+    fdu_status st;
+    if ((st = m->alloc(base, nt * kTile + noff))) return st;
+    T.perm = base;
+    T.voff = base + nt * kTile;
+    T.eoff = T.voff + nt + 1;
+    T.gvoff = T.eoff + nt + 1;
+    T.geoff = T.gvoff + ns + 1;
+    launch_tile_count(S, T, T.voff + 1, T.eoff + 1, T.gvoff + 1, T.geoff + 1, nullptr);
+    CK_LAUNCH();
+    std::vector<int32_t> h(noff);
+    CK(cudaMemcpy(h.data(), T.voff, noff * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    int32_t *hv = h.data(), *he = hv + nt + 1, *gv = he + nt + 1, *ge = gv + ns + 1;
+    for (int64_t t = 1; t <= nt; ++t) {
+        if (hv[t] < 0 || he[t] < 0) return FDU_OK;
+        T.smem = std::max(T.smem, 32 * hv[t] + 16 * he[t]);
+    }
+    hv[0] = he[0] = gv[0] = ge[0] = 0;
+    for (int32_t *p : {hv, he})
+        for (int64_t t = 1; t <= nt; ++t) {
+            if (p[t] > INT32_MAX - p[t - 1]) return FDU_OK;
+            p[t] += p[t - 1];
+        }
+    for (int32_t *p : {gv, ge})
+        for (int64_t t = 1; t <= ns; ++t) p[t] += p[t - 1];
+    if (T.smem > kMaxBytes) return FDU_OK;
+    CK(cudaMemcpy(T.voff, h.data(), noff * sizeof(int32_t), cudaMemcpyHostToDevice));
+    int32_t *list = nullptr;
+    ushort4 *pos = nullptr;
+    float4 *wt = nullptr;
+    if ((st = m->alloc(list, hv[nt] + (int64_t)he[nt]))) return st;
+    if ((st = m->alloc(pos, kSell * (gv[ns] + (int64_t)ge[ns])))) return st;
+    if ((st = m->alloc(wt, kSell * (2 * (int64_t)gv[ns] + ge[ns])))) return st;
+    T.vlist = list;
+    T.elist = list + hv[nt];
+    T.vpos = pos;
+    T.epos = pos + (int64_t)kSell * gv[ns];
+    T.wf = wt;
+    T.wg = wt + (int64_t)kSell * gv[ns];
+    T.we = wt + (int64_t)kSell * 2 * gv[ns];
+    launch_tile_fill(S, T, nullptr);
+    CK_LAUNCH();
+    CK(cudaDeviceSynchronize());
+    m->tile32 = T;
+    return FDU_OK;
+}
+
 DivArgs div_args(fdu_mesh *m, int prec, int fin);
 fdu_status build_dw_tables(fdu_mesh *m) {
     const int64_t ne = m->ne_act, nr = std::max<int64_t>(m->n_real, 1);
@@ -418,7 +481,8 @@ fdu_status upload_tables(fdu_mesh *m) {
     m->nsteps = reinterpret_cast<unsigned long long *>(m->tstate + 3);
     m->wide = reinterpret_cast<int *>(m->tstate + 4);
     CK(cudaMemset(m->wn, 0, 4 * nv * sizeof(double)));
-    return build_dw_tables(m);
+    if ((st = build_dw_tables(m))) return st;
+    return build_tiles(m);
 }
 
 // Precision 48: the FP64 state pipeline (FP64 divergence and stage) with
@@ -571,6 +635,7 @@ void enqueue_stages(fdu_mesh *m, int prec, double dt, const double *dt_dev, cuda
         a.dt_dev = dt_dev;
         timed(m, kd + 1, prof, s, [&] {
             if (f64) launch_div_f64(a, stage, s);
+            else if (m->tile32.smem) launch_div_f32_tiles(a, m->tile32, stage, s);
             else launch_div_f32(a, stage, s);
         });
         if (m->n_ghost > 0) {
@@ -1137,6 +1202,7 @@ fdu_status fdu_residual(fdu_mesh *m, int precision, double *dwdt, int on_device,
     a.out_map = m->new2old;
     timed(m, kd + 1, true, s, [&] {
         if (f64) launch_div_f64(a, 0, s);
+        else if (m->tile32.smem) launch_div_f32_tiles(a, m->tile32, 0, s);
         else launch_div_f32(a, 0, s);
     });
     CK_LAUNCH();

@@ -282,7 +282,7 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
         const float4 *__restrict__ rd = static_cast<const float4 *>(A.r);
         dot2 sx{0.0f, 0.0f}, sy = sx, sz = sx, sw = sx;
         const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = __ldg(A.slice_eoff + sl + 1);
-#pragma unroll 4
+#pragma unroll 6
         for (int64_t p = b; p < e; p += kSell) {
             const int32_t k = tld<MODE>(A.eid + p);
             const float2 wq = tld<MODE>(we2 + p);
@@ -782,13 +782,343 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) edge_flux_guard_kernel(const __
     dwa::clear_wide(A, e);
     edge_flux_guard_body(A, e, dwa::Stage{stage + threadIdx.x, kEdgeBlock}, stage_is_wide(A.wide, A.wide_in));
 }
+// At most 80 registers (6 blocks, 24 warps per SM): with the 56 the compiler
+// takes when left alone fewer gathers are in flight (precision 48 0.139 against
+// 0.120 ms at 250k vertices; 64 registers 0.123, 40 with 9 blocks 0.139).
 template <int MODE, int KIND>
-__global__ void __launch_bounds__(kDivBlock) div_f64_kernel(const __grid_constant__ DivArgs A) {
+__global__ void __launch_bounds__(kDivBlock, 6) div_f64_kernel(const __grid_constant__ DivArgs A) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= A.n_real) return;
     if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;  // adaptive run already at t_end
     div_f64_any<MODE, KIND>(A, v, KIND == kDivGuard && stage_is_wide(A.wide, A.wide_in));
 }
+// ------------------------------------------------------------------ divergence tiles
+constexpr int kTileThreads = 256;  // threads of the tile-building kernels
+constexpr int kTileSteps = 96;     // longest slice whose entries are scheduled over the banks
+// The real entries of vertex v in a SELL layout (natural order): J vertex
+// entries (padding names v itself, which is never its own neighbour) and K edge
+// entries (padding repeats the first).
+struct TileRow {
+    int64_t vb, eb;
+    int J, K;
+};
+__device__ __forceinline__ TileRow tile_row(const TileSource &S, int64_t v) {
+    const int64_t sl = v / kSell;
+    const int lane = (int)(v % kSell);
+    TileRow r;
+    r.vb = S.slice_voff[sl] + lane;
+    r.eb = S.slice_eoff[sl] + lane;
+    const int64_t ve = S.slice_voff[sl + 1], ee = S.slice_eoff[sl + 1];
+    r.J = r.K = 0;
+    for (int64_t p = r.vb; p < ve; p += kSell) r.J += S.vid[p] != (int32_t)v;
+    for (int64_t p = r.eb; p < ee; p += kSell) r.K += p == r.eb || S.eid[p] != S.eid[r.eb];
+    return r;
+}
+// One tile's shared state while it is built.
+struct TileWork {
+    int32_t hash[2 * kTileMaxE], list[kTileMaxE];
+    int count;
+    int J[kTile], K[kTile];  // by position
+    unsigned char left[kTile][8];           // entries of a lane still to place, by bank
+    unsigned char bank[kTileSteps][kTile];  // bank of the entry a lane takes at each step (8: none)
+};
+// The tile's distinct vertices (edges = false; with the tile's own) or edges:
+// a hash table in shared memory, compacted and sorted.  Returns the count, -1
+// beyond the capacity.  Every thread of the block calls it.
+__device__ int tile_unique(TileWork &W, const TileSource &S, int64_t v0, int nvt, bool edges) {
+    const int most = edges ? kTileMaxE : kTileMaxV, cap = 2 * most;
+    for (int i = threadIdx.x; i < cap; i += kTileThreads) W.hash[i] = -1;
+    if (threadIdx.x == 0) W.count = 0;
+    __syncthreads();
+    auto insert = [&](int32_t id) {
+        unsigned h = ((unsigned)id * 2654435761u) & (unsigned)(cap - 1);
+        while (*(volatile int *)&W.count <= most) {  // at most half of the slots are ever taken, plus one per thread
+            const int32_t old = atomicCAS(W.hash + h, -1, id);
+            if (old == -1) atomicAdd(&W.count, 1);
+            if (old == -1 || old == id) break;
+            h = (h + 1) & (unsigned)(cap - 1);
+        }
+    };
+    for (int i = threadIdx.x; i < nvt; i += kTileThreads) {
+        const TileRow r = tile_row(S, v0 + i);
+        if (edges) {
+            for (int j = 0; j < r.K; ++j) insert(S.eid[r.eb + (int64_t)kSell * j]);
+        } else {
+            insert((int32_t)(v0 + i));
+            for (int j = 0; j < r.J; ++j) insert(S.vid[r.vb + (int64_t)kSell * j]);
+        }
+    }
+    __syncthreads();
+    const int total = W.count;
+    __syncthreads();
+    if (total > most) return -1;
+    if (threadIdx.x == 0) W.count = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < cap; i += kTileThreads)
+        if (W.hash[i] >= 0) W.list[atomicAdd(&W.count, 1)] = W.hash[i];
+    int m = 1;
+    while (m < total) m <<= 1;
+    __syncthreads();
+    for (int i = total + (int)threadIdx.x; i < m; i += kTileThreads) W.list[i] = INT32_MAX;
+    __syncthreads();
+    for (int k = 2; k <= m; k <<= 1)  // bitonic sort
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int i = threadIdx.x; i < m; i += kTileThreads) {
+                const int q = i ^ j;
+                if (q > i) {
+                    const int32_t a = W.list[i], c = W.list[q];
+                    if ((a > c) == ((i & k) == 0)) {
+                        W.list[i] = c;
+                        W.list[q] = a;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    return total;
+}
+__device__ unsigned short tile_position(const int32_t *list, int n, int32_t id) {
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (list[mid] < id) lo = mid + 1;
+        else hi = mid;
+    }
+    return (unsigned short)lo;
+}
+__global__ void __launch_bounds__(kTileThreads)
+    tile_count_kernel(TileSource S, TileTables T, int32_t *nv, int32_t *ne, int32_t *gv, int32_t *ge) {
+    extern __shared__ int tile_work[];
+    TileWork &W = *reinterpret_cast<TileWork *>(tile_work);
+    __shared__ int key[kTile];
+    const int64_t t = blockIdx.x, v0 = t * kTile;
+    const int nvt = (int)min((int64_t)kTile, S.n_real - v0), i = threadIdx.x;
+    TileRow r{0, 0, 0, 0};
+    if (i < kTile) {
+        if (i < nvt) r = tile_row(S, v0 + i);
+        key[i] = i < nvt ? (r.J << 16) | r.K : -1;
+    }
+    __syncthreads();
+    if (i < kTile) {  // decreasing (J, K), ties in vertex order
+        int rank = 0;
+        for (int q = 0; q < kTile; ++q) rank += key[q] > key[i] || (key[q] == key[i] && q < i);
+        W.J[rank] = r.J;
+        W.K[rank] = r.K;
+        T.perm[v0 + rank] = i < nvt ? (int32_t)(v0 + i) : -1;
+    }
+    __syncthreads();
+    if (i < kTile / kSell) {
+        int mj = 0, mk = 0;
+        for (int l = 0; l < kSell; ++l) {
+            mj = max(mj, W.J[i * kSell + l]);
+            mk = max(mk, W.K[i * kSell + l]);
+        }
+        gv[t * (kTile / kSell) + i] = (mj + 3) / 4;
+        ge[t * (kTile / kSell) + i] = (mk + 3) / 4;
+    }
+    const int a = tile_unique(W, S, v0, nvt, false);
+    __syncthreads();
+    const int c = tile_unique(W, S, v0, nvt, true);
+    if (i == 0) {
+        nv[t] = a;
+        ne[t] = c;
+    }
+}
+// Order of a slice's entries over its steps.  A 16-byte shared-memory read is
+// served eight lanes at a time, and positions equal modulo 8 fall on the same
+// banks, so each group of eight lanes takes entries of different banks where it
+// can: per step, each lane (starting from another one each time) takes from its
+// fullest bank that no lane before it took, waits a step if it has some to
+// spare, and conflicts otherwise.  One thread per group; W.left holds the lanes'
+// entry counts by bank.
+__device__ void tile_schedule(TileWork &W, int group, int steps) {
+    const int l0 = 8 * group;
+    int rest[8];
+    for (int l = 0; l < 8; ++l) {
+        rest[l] = 0;
+        for (int c = 0; c < 8; ++c) rest[l] += W.left[l0 + l][c];
+    }
+    for (int s = 0; s < steps; ++s) {
+        unsigned used = 0;
+        for (int q = 0; q < 8; ++q) {
+            const int l = (q + s) & 7;
+            int best = 8, any = 8;
+            for (int c = 0; c < 8; ++c) {
+                const int n = W.left[l0 + l][c];
+                if (n == 0) continue;
+                if (any == 8 || n > W.left[l0 + l][any]) any = c;
+                if (!(used >> c & 1u) && (best == 8 || n > W.left[l0 + l][best])) best = c;
+            }
+            if (best == 8 && rest[l] >= steps - s) best = any;
+            W.bank[s][l0 + l] = (unsigned char)best;
+            if (best == 8) continue;
+            used |= 1u << best;
+            --W.left[l0 + l][best];
+            --rest[l];
+        }
+    }
+}
+// Writes one lane's entries (n of them, `entry(j)` the position of the j-th in
+// the tile's list) as put(step, position, entry index or -1) over the slice's
+// steps: in list order, or by W.bank where `scheduled`.  A step without an entry
+// repeats the lane's first with weight 0, as the SELL padding does, so that a
+// non-finite flux reaches only the vertices whose stencil holds it.
+template <class E, class P>
+__device__ __forceinline__ void tile_write(const TileWork &W, int lane, int n, int steps, bool scheduled, E &&entry,
+                                           P &&put) {
+    int cur[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int s = 0; s < steps; ++s) {
+        int j = s < n ? s : -1;
+        if (scheduled) {
+            const int c = W.bank[s][lane];
+            j = -1;
+            if (c < 8) {
+                int q = cur[c];
+                while ((entry(q) & 7) != c) ++q;
+                cur[c] = q + 1;
+                j = q;
+            }
+        }
+        put(s, n > 0 ? entry(j < 0 ? 0 : j) : 0, j);
+    }
+}
+__global__ void __launch_bounds__(kTileThreads) tile_fill_kernel(TileSource S, TileTables T) {
+    extern __shared__ int tile_work[];
+    TileWork &W = *reinterpret_cast<TileWork *>(tile_work);
+    const int64_t t = blockIdx.x, v0 = t * kTile;
+    const int nvt = (int)min((int64_t)kTile, S.n_real - v0), i = threadIdx.x;
+    const int32_t v = i < kTile ? T.perm[v0 + i] : -1;
+    const TileRow r = v >= 0 ? tile_row(S, v) : TileRow{0, 0, 0, 0};
+    const int64_t sl = t * (kTile / kSell) + i / kSell, lane = i % kSell;
+    for (int part = 0; part < 2; ++part) {
+        const int32_t *ids = part ? S.eid : S.vid;
+        const int64_t b = part ? r.eb : r.vb;
+        const int cnt = part ? r.K : r.J;
+        const int32_t *goff = part ? T.geoff : T.gvoff;
+        const int n = tile_unique(W, S, v0, nvt, part != 0);
+        int32_t *list = part ? T.elist + T.eoff[t] : T.vlist + T.voff[t];
+        for (int q = i; q < n; q += kTileThreads) list[q] = W.list[q];
+        auto entry = [&](int j) { return tile_position(W.list, n, ids[b + (int64_t)kSell * j]); };
+        const int steps = i < kTile ? 4 * (goff[sl + 1] - goff[sl]) : 0;
+        const bool scheduled = steps <= kTileSteps && cnt < 256;
+        if (i < kTile) {
+            for (int c = 0; c < 8; ++c) W.left[i][c] = 0;
+            if (scheduled)
+                for (int j = 0; j < cnt; ++j) ++W.left[i][entry(j) & 7];
+        }
+        __syncthreads();
+        if (i < kTile && scheduled && i % 8 == 0) tile_schedule(W, i / 8, steps);
+        __syncthreads();
+        if (i < kTile) {
+            const int64_t g0 = goff[sl];
+            unsigned short *pos = reinterpret_cast<unsigned short *>(part ? T.epos : T.vpos);
+            float *wa = reinterpret_cast<float *>(part ? T.we : T.wf), *wb = reinterpret_cast<float *>(T.wg);
+            tile_write(W, i, cnt, steps, scheduled, entry, [&](int s, unsigned short p, int j) {
+                const int64_t q = 4 * ((g0 + s / 4) * kSell + lane) + s % 4;
+                const int64_t src = b + (int64_t)kSell * j;
+                pos[q] = p;
+                wa[q] = j >= 0 ? (part ? S.we : S.wf)[src] : 0.0f;
+                if (!part) wb[q] = j >= 0 ? S.wg[src] : 0.0f;
+            });
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ void cp_async16(void *smem, const void *g) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(g)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ ushort4 ld_stream(const ushort4 *p) {
+    ushort4 v;
+    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u16 {%0, %1, %2, %3}, [%4];"
+        : "=h"(v.x), "=h"(v.y), "=h"(v.z), "=h"(v.w)
+        : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_stream(const float4 *p) {
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
+    return v;
+}
+
+// FP32 divergence (+ stage) over tiles: one block copies its tile's fluxes into
+// shared memory, then each thread walks the entries of one vertex there.
+//
+// What bounds it: the table stream (about 510 bytes per vertex from DRAM, 60 %
+// of the measured HBM rate) and its latency; the reads of the staged fluxes
+// take half of the shared-memory cycles.  Gathering every entry from global
+// memory (div_f32_kernel) costs 12 L1 wavefronts where 4 would carry the data
+// (L1 76 % busy) and 8 and 12 bytes per entry with full ids: 0.0532 ms in the
+// stage and 0.066 ms for the residual alone at 250k vertices, here 0.0417 and
+// 0.0354 ms.  On the way: the same tables staged 0.050 (16-bit positions),
+// entries in groups of four 0.0467, banks scheduled (tile_schedule) 0.0445, 73
+// registers and 7 blocks per SM instead of 64 and 8 0.0417.  Tiles of 256
+// (0.054), table groups read ahead explicitly (0.044 to 0.064) and 6 or 9
+// blocks per SM (0.052, 0.045) are slower.
+template <int MODE>
+__global__ void __launch_bounds__(kTile, 7) div_f32_tile_kernel(const __grid_constant__ DivArgs A,
+                                                                 const __grid_constant__ TileTables T) {
+    extern __shared__ float4 sm[];
+    if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;
+    const int64_t t = blockIdx.x;
+    const int v0 = __ldg(T.voff + t), nvt = __ldg(T.voff + t + 1) - v0;
+    const int e0 = __ldg(T.eoff + t), net = __ldg(T.eoff + t + 1) - e0;
+    float4 *sf = sm, *sg = sm + nvt, *sr = sm + 2 * nvt;
+    const float4 *__restrict__ F = static_cast<const float4 *>(A.F);
+    const float4 *__restrict__ r = static_cast<const float4 *>(A.r);
+    for (int i = threadIdx.x; i < net; i += kTile) cp_async16(sr + i, r + __ldg(T.elist + e0 + i));
+    for (int i = threadIdx.x; i < nvt; i += kTile) {
+        const int64_t j = __ldg(T.vlist + v0 + i);
+        cp_async16(sf + i, F + 2 * j);
+        cp_async16(sg + i, F + 2 * j + 1);
+    }
+    const int64_t sl = t * (kTile / kSell) + threadIdx.x / kSell;
+    const int lane = threadIdx.x % kSell;
+    const int32_t v = __ldg(T.perm + t * kTile + threadIdx.x);
+    const int gb = __ldg(T.gvoff + sl), ge = __ldg(T.gvoff + sl + 1);
+    const int hb = __ldg(T.geoff + sl), he = __ldg(T.geoff + sl + 1);
+    cp_async_wait();
+    __syncthreads();
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto vert = [&](int j, float a, float c) {
+        const float4 f = sf[j], g = sg[j];
+        acc.x = fmaf(a, f.x, fmaf(c, g.x, acc.x));
+        acc.y = fmaf(a, f.y, fmaf(c, g.y, acc.y));
+        acc.z = fmaf(a, f.z, fmaf(c, g.z, acc.z));
+        acc.w = fmaf(a, f.w, fmaf(c, g.w, acc.w));
+    };
+#pragma unroll 2
+    for (int g = gb; g < ge; ++g) {
+        const ushort4 j = ld_stream(T.vpos + (int64_t)g * kSell + lane);
+        const float4 a = ld_stream(T.wf + (int64_t)g * kSell + lane), c = ld_stream(T.wg + (int64_t)g * kSell + lane);
+        vert(j.x, a.x, c.x);
+        vert(j.y, a.y, c.y);
+        vert(j.z, a.z, c.z);
+        vert(j.w, a.w, c.w);
+    }
+    auto edge = [&](int k, float a) {
+        const float4 q = sr[k];
+        acc.x = fmaf(a, q.x, acc.x);
+        acc.y = fmaf(a, q.y, acc.y);
+        acc.z = fmaf(a, q.z, acc.z);
+        acc.w = fmaf(a, q.w, acc.w);
+    };
+#pragma unroll 4
+    for (int h = hb; h < he; ++h) {
+        const ushort4 k = ld_stream(T.epos + (int64_t)h * kSell + lane);
+        const float4 a = ld_stream(T.we + (int64_t)h * kSell + lane);
+        edge(k.x, a.x);
+        edge(k.y, a.y);
+        edge(k.z, a.z);
+        edge(k.w, a.w);
+    }
+    if (v >= 0) div_f32_finish<MODE>(A, v, acc);
+}
+
 // Folded tables of the double-word divergence (launch_fold_tables); thread i
 // serves SELL position i.  Entries and sums in the order of the SELL lists,
 // rounded one by one.
@@ -1117,6 +1447,23 @@ void launch_div_f32(const DivArgs &a, int mode, cudaStream_t s) {
         case 1: div_f32_kernel<1><<<g, kDivBlock, 0, s>>>(a); break;
         case 2: div_f32_kernel<2><<<g, kDivBlock, 0, s>>>(a); break;
         default: div_f32_kernel<3><<<g, kDivBlock, 0, s>>>(a); break;
+    }
+}
+void launch_tile_count(const TileSource &S, const TileTables &T, int32_t *nv, int32_t *ne, int32_t *gv, int32_t *ge,
+                       cudaStream_t s) {
+    if (T.ntiles > 0)
+        tile_count_kernel<<<(unsigned)T.ntiles, kTileThreads, sizeof(TileWork), s>>>(S, T, nv, ne, gv, ge);
+}
+void launch_tile_fill(const TileSource &S, const TileTables &T, cudaStream_t s) {
+    if (T.ntiles > 0) tile_fill_kernel<<<(unsigned)T.ntiles, kTileThreads, sizeof(TileWork), s>>>(S, T);
+}
+void launch_div_f32_tiles(const DivArgs &a, const TileTables &t, int mode, cudaStream_t s) {
+    const unsigned g = (unsigned)t.ntiles;
+    switch (mode) {
+        case 0: div_f32_tile_kernel<0><<<g, kTile, t.smem, s>>>(a, t); break;
+        case 1: div_f32_tile_kernel<1><<<g, kTile, t.smem, s>>>(a, t); break;
+        case 2: div_f32_tile_kernel<2><<<g, kTile, t.smem, s>>>(a, t); break;
+        default: div_f32_tile_kernel<3><<<g, kTile, t.smem, s>>>(a, t); break;
     }
 }
 void launch_check_rows(const double *w, int64_t n, unsigned long long *bad, cudaStream_t s) {

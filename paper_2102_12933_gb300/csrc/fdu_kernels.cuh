@@ -99,6 +99,39 @@ struct DivArgs {
     unsigned long long *limited; // vertices whose stage update the safeguard scaled
 };
 
+// ---- Divergence tiles.  A tile is kTile consecutive vertices (internal order).
+// The distinct vertices and edges of its stencils are listed once (ascending
+// ids), a block copies their fluxes into shared memory, and the stencil entries
+// name them by 16-bit position in those lists.  Inside a tile the vertices are
+// ordered by decreasing stencil size (perm), 32 to a slice; a slice's entries
+// are stored in groups of four per lane (four positions, four weights: 8- and
+// 16-byte loads), each slice padded to its longest list with weight 0.
+constexpr int kTile = 128;
+constexpr int kTileMaxV = 1024, kTileMaxE = 2048;  // capacity of a tile's lists
+// Source of the tiles: a SELL layout of the divergence tables.
+struct TileSource {
+    int64_t n_real;
+    const int64_t *slice_voff, *slice_eoff;
+    const int32_t *vid, *eid;
+    const float *wf, *wg, *we;
+};
+struct TileTables {
+    int64_t ntiles;
+    int smem;                    // staging bytes of the largest tile (0: no tiles)
+    int32_t *perm;               // [ntiles * kTile] vertex at each position (-1 past the last)
+    int32_t *voff, *eoff;        // [ntiles + 1] start of each tile's lists
+    int32_t *vlist, *elist;      // vertex and edge ids
+    int32_t *gvoff, *geoff;      // [ntiles * kTile / kSell + 1] first entry group of each slice
+    ushort4 *vpos, *epos;        // [groups][kSell] positions in the tile's lists
+    float4 *wf, *wg, *we;        // [groups][kSell] weights
+};
+// Sizes of the tiles' lists (nv, ne; -1 where a tile exceeds the capacity) and
+// of the slices' entry groups (gv, ge), and the positions' order (T.perm).
+void launch_tile_count(const TileSource &S, const TileTables &T, int32_t *nv, int32_t *ne, int32_t *gv, int32_t *ge,
+                       cudaStream_t s);
+// Lists, positions and weights (the offsets are in place).
+void launch_tile_fill(const TileSource &S, const TileTables &T, cudaStream_t s);
+
 // F[v] = (f, g) of w[v]; Q (optional) = Roe records (sqrt rho, sqrt rho u, sqrt rho v, sqrt rho H)
 // wide (optional): slot 0 of the WideFlags for vertices below n_real, kWideGhost for the others
 void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q = nullptr,
@@ -120,6 +153,7 @@ void launch_coef_dw(const double *coef, float4 *coefdw, int64_t ne, int *bad, cu
 void launch_dw_check(int op, const double *x, const double *y, double *z, int64_t n, cudaStream_t s);
 void launch_div_f64(const DivArgs &a, int mode, cudaStream_t s);
 void launch_div_f32(const DivArgs &a, int mode, cudaStream_t s);
+void launch_div_f32_tiles(const DivArgs &a, const TileTables &t, int mode, cudaStream_t s);
 // *bad = min(*bad, first row of w[n][4] with rho <= 0 or a non-finite value)
 void launch_check_rows(const double *w, int64_t n, unsigned long long *bad, cudaStream_t s);
 void launch_permute_rows(const double *in, double *out, const int32_t *map, int64_t n, bool gather, cudaStream_t s);
