@@ -128,14 +128,33 @@ struct fdu_mesh {
     std::vector<cudaEvent_t> prof_ev[6];
     size_t prof_used[6] = {0, 0, 0, 0, 0, 0};
 
+    // Device memory of the mesh, freed with it.  Requests up to kSmall share
+    // chunks: a cudaMalloc takes tens of microseconds, and a small mesh makes
+    // about fifty requests.
+    static constexpr size_t kSmall = 256 << 10, kChunk = 4 << 20, kAlign = 256;
+    char *chunk = nullptr;
+    size_t chunk_left = 0;
     template <class T>
     fdu_status alloc(T *&p, size_t count) {
         p = nullptr;
         if (count == 0) count = 1;
+        const size_t bytes = (count * sizeof(T) + kAlign - 1) / kAlign * kAlign;
         void *q = nullptr;
-        cudaError_t e = cudaMalloc(&q, count * sizeof(T));
-        if (e != cudaSuccess) return set_err(FDU_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-        allocs.push_back(q);
+        if (bytes > kSmall || bytes > chunk_left) {
+            const size_t take = bytes > kSmall ? bytes : kChunk;
+            cudaError_t e = cudaMalloc(&q, take);
+            if (e != cudaSuccess) return set_err(FDU_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+            allocs.push_back(q);
+            if (bytes <= kSmall) {
+                chunk = static_cast<char *>(q);
+                chunk_left = take;
+            }
+        }
+        if (bytes <= kSmall) {
+            q = chunk;
+            chunk += bytes;
+            chunk_left -= bytes;
+        }
         device_bytes += (int64_t)(count * sizeof(T));
         p = static_cast<T *>(q);
         return FDU_OK;

@@ -816,10 +816,13 @@ __device__ __forceinline__ TileRow tile_row(const TileSource &S, int64_t v) {
 }
 // One tile's shared state while it is built.
 struct TileWork {
-    int32_t hash[2 * kTileMaxE], list[kTileMaxE];
+    union {
+        int32_t hash[2 * kTileMaxE];
+        unsigned short pos[kTileSteps][kTile];  // a lane's positions in the tile's list, in list order
+    };
+    int32_t list[kTileMaxE];
     int count;
-    int J[kTile], K[kTile];  // by position
-    unsigned char left[kTile][8];           // entries of a lane still to place, by bank
+    int J[kTile], K[kTile];                 // by position
     unsigned char bank[kTileSteps][kTile];  // bank of the entry a lane takes at each step (8: none)
 };
 // The tile's distinct vertices (edges = false; with the tile's own) or edges:
@@ -839,13 +842,15 @@ __device__ int tile_unique(TileWork &W, const TileSource &S, int64_t v0, int nvt
             h = (h + 1) & (unsigned)(cap - 1);
         }
     };
-    for (int i = threadIdx.x; i < nvt; i += kTileThreads) {
-        const TileRow r = tile_row(S, v0 + i);
+    constexpr int kShare = kTileThreads / kTile;  // threads that share a vertex's entries
+    const int i0 = threadIdx.x % kTile, j0 = threadIdx.x / kTile;
+    if (i0 < nvt) {
+        const TileRow r = tile_row(S, v0 + i0);
         if (edges) {
-            for (int j = 0; j < r.K; ++j) insert(S.eid[r.eb + (int64_t)kSell * j]);
+            for (int j = j0; j < r.K; j += kShare) insert(S.eid[r.eb + (int64_t)kSell * j]);
         } else {
-            insert((int32_t)(v0 + i));
-            for (int j = 0; j < r.J; ++j) insert(S.vid[r.vb + (int64_t)kSell * j]);
+            if (j0 == 0) insert((int32_t)(v0 + i0));
+            for (int j = j0; j < r.J; j += kShare) insert(S.vid[r.vb + (int64_t)kSell * j]);
         }
     }
     __syncthreads();
@@ -927,60 +932,45 @@ __global__ void __launch_bounds__(kTileThreads)
 // Order of a slice's entries over its steps.  A 16-byte shared-memory read is
 // served eight lanes at a time, and positions equal modulo 8 fall on the same
 // banks, so each group of eight lanes takes entries of different banks where it
-// can: per step, each lane (starting from another one each time) takes from its
-// fullest bank that no lane before it took, waits a step if it has some to
-// spare, and conflicts otherwise.  One thread per group; W.left holds the lanes'
-// entry counts by bank.
-__device__ void tile_schedule(TileWork &W, int group, int steps) {
-    const int l0 = 8 * group;
+// can: per step, each lane (starting from another one each time) takes the next
+// bank, from its own place in a rotation, that it has entries of and no lane
+// before it took; otherwise it waits a step if it has some to spare, or takes
+// a taken one.  One thread per group; n[l] = entries of lane l, left[l] = their
+// counts by bank, a byte each.
+__device__ void tile_schedule(TileWork &W, int group, int steps, const int *n) {
+    unsigned long long left[8];
+    unsigned has[8];
     int rest[8];
+#pragma unroll
     for (int l = 0; l < 8; ++l) {
-        rest[l] = 0;
-        for (int c = 0; c < 8; ++c) rest[l] += W.left[l0 + l][c];
+        left[l] = 0;
+        rest[l] = n[8 * group + l];
+        for (int j = 0; j < rest[l]; ++j) left[l] += 1ull << (8 * (W.pos[j][8 * group + l] & 7));
+        has[l] = 0;
+        for (int c = 0; c < 8; ++c) has[l] |= (unsigned)((left[l] >> (8 * c) & 0xff) != 0) << c;
     }
-    for (int s = 0; s < steps; ++s) {
-        unsigned used = 0;
-        for (int q = 0; q < 8; ++q) {
-            const int l = (q + s) & 7;
-            int best = 8, any = 8;
-            for (int c = 0; c < 8; ++c) {
-                const int n = W.left[l0 + l][c];
-                if (n == 0) continue;
-                if (any == 8 || n > W.left[l0 + l][any]) any = c;
-                if (!(used >> c & 1u) && (best == 8 || n > W.left[l0 + l][best])) best = c;
-            }
-            if (best == 8 && rest[l] >= steps - s) best = any;
-            W.bank[s][l0 + l] = (unsigned char)best;
-            if (best == 8) continue;
-            used |= 1u << best;
-            --W.left[l0 + l][best];
-            --rest[l];
-        }
-    }
-}
-// Writes one lane's entries (n of them, `entry(j)` the position of the j-th in
-// the tile's list) as put(step, position, entry index or -1) over the slice's
-// steps: in list order, or by W.bank where `scheduled`.  A step without an entry
-// repeats the lane's first with weight 0, as the SELL padding does, so that a
-// non-finite flux reaches only the vertices whose stencil holds it.
-template <class E, class P>
-__device__ __forceinline__ void tile_write(const TileWork &W, int lane, int n, int steps, bool scheduled, E &&entry,
-                                           P &&put) {
-    int cur[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int s = 0; s < steps; ++s) {
-        int j = s < n ? s : -1;
-        if (scheduled) {
-            const int c = W.bank[s][lane];
-            j = -1;
-            if (c < 8) {
-                int q = cur[c];
-                while ((entry(q) & 7) != c) ++q;
-                cur[c] = q + 1;
-                j = q;
+    for (int s0 = 0; s0 < steps; s0 += 8)
+#pragma unroll
+        for (int ds = 0; ds < 8; ++ds) {
+            const int s = s0 + ds;
+            if (s >= steps) break;
+            unsigned used = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int l = (q + ds) & 7, first = (s + l) & 7;
+                unsigned m = has[l] & ~used;
+                if (m == 0 && rest[l] >= steps - s) m = has[l];
+                int c = 8;
+                if (m) {
+                    c = (__ffs((m | m << 8) >> first) - 1 + first) & 7;
+                    used |= 1u << c;
+                    left[l] -= 1ull << (8 * c);
+                    if ((left[l] >> (8 * c) & 0xff) == 0) has[l] &= ~(1u << c);
+                    --rest[l];
+                }
+                W.bank[s][8 * group + l] = (unsigned char)c;
             }
         }
-        put(s, n > 0 ? entry(j < 0 ? 0 : j) : 0, j);
-    }
 }
 __global__ void __launch_bounds__(kTileThreads) tile_fill_kernel(TileSource S, TileTables T) {
     extern __shared__ int tile_work[];
@@ -998,28 +988,47 @@ __global__ void __launch_bounds__(kTileThreads) tile_fill_kernel(TileSource S, T
         const int n = tile_unique(W, S, v0, nvt, part != 0);
         int32_t *list = part ? T.elist + T.eoff[t] : T.vlist + T.voff[t];
         for (int q = i; q < n; q += kTileThreads) list[q] = W.list[q];
-        auto entry = [&](int j) { return tile_position(W.list, n, ids[b + (int64_t)kSell * j]); };
-        const int steps = i < kTile ? 4 * (goff[sl + 1] - goff[sl]) : 0;
-        const bool scheduled = steps <= kTileSteps && cnt < 256;
+        const int64_t g0 = i < kTile ? goff[sl] : 0;
+        const int steps = i < kTile ? 4 * (int)(goff[sl + 1] - g0) : 0;
+        const bool scheduled = steps <= kTileSteps;  // the same for the lanes of a slice
+        int *count = part ? W.K : W.J;
+        __syncthreads();  // the hash table's memory holds positions from here
         if (i < kTile) {
-            for (int c = 0; c < 8; ++c) W.left[i][c] = 0;
+            count[i] = cnt;
             if (scheduled)
-                for (int j = 0; j < cnt; ++j) ++W.left[i][entry(j) & 7];
+                for (int j = 0; j < cnt; ++j) W.pos[j][i] = tile_position(W.list, n, ids[b + (int64_t)kSell * j]);
         }
         __syncthreads();
-        if (i < kTile && scheduled && i % 8 == 0) tile_schedule(W, i / 8, steps);
+        if (i < kTile && scheduled && i % 8 == 0) tile_schedule(W, i / 8, steps, count);
         __syncthreads();
         if (i < kTile) {
-            const int64_t g0 = goff[sl];
+            // a step without an entry repeats the lane's first with weight 0, as
+            // the SELL padding does, so that a non-finite flux reaches only the
+            // vertices whose stencils hold it
             unsigned short *pos = reinterpret_cast<unsigned short *>(part ? T.epos : T.vpos);
             float *wa = reinterpret_cast<float *>(part ? T.we : T.wf), *wb = reinterpret_cast<float *>(T.wg);
-            tile_write(W, i, cnt, steps, scheduled, entry, [&](int s, unsigned short p, int j) {
-                const int64_t q = 4 * ((g0 + s / 4) * kSell + lane) + s % 4;
-                const int64_t src = b + (int64_t)kSell * j;
+            const float *sa = part ? S.we : S.wf;
+            unsigned char cur[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            for (int s = 0; s < steps; ++s) {
+                int j = s < cnt ? s : -1;
+                unsigned short p = 0;
+                if (scheduled) {
+                    const int c = W.bank[s][i];
+                    j = -1;
+                    if (c < 8) {
+                        j = cur[c];
+                        while ((W.pos[j][i] & 7) != c) ++j;
+                        cur[c] = (unsigned char)(j + 1);
+                    }
+                    if (cnt > 0) p = W.pos[j < 0 ? 0 : j][i];
+                } else if (cnt > 0) {
+                    p = tile_position(W.list, n, ids[b + (int64_t)kSell * (j < 0 ? 0 : j)]);
+                }
+                const int64_t q = 4 * ((g0 + s / 4) * kSell + lane) + s % 4, src = b + (int64_t)kSell * j;
                 pos[q] = p;
-                wa[q] = j >= 0 ? (part ? S.we : S.wf)[src] : 0.0f;
+                wa[q] = j >= 0 ? sa[src] : 0.0f;
                 if (!part) wb[q] = j >= 0 ? S.wg[src] : 0.0f;
-            });
+            }
         }
         __syncthreads();
     }
