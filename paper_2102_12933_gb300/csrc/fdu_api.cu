@@ -288,15 +288,27 @@ void stencil_gaps(const double xi[6], float g[4]) {
 fdu_status build_tiles(fdu_mesh *m) {
     constexpr int kSlices = kTile / kSell;
     constexpr int kMaxBytes = 48 * 1024;  // shared memory of a launch without opt-in
+    if (m->n_real == 0) return FDU_OK;
+    std::vector<int32_t> start;
+    for (int64_t v = 0; v < m->n_real;) {  // a mesh of a batch holds consecutive vertices
+        int64_t end = m->n_real;
+        if (m->n_comp > 0) {
+            const auto c = std::upper_bound(m->comp_voff.begin(), m->comp_voff.end(), (int64_t)m->T.v_new2old[v]);
+            end = v + (*c - *(c - 1));
+        }
+        for (; v < end; v = std::min<int64_t>(end, v + kTile)) start.push_back((int32_t)v);
+    }
+    start.push_back((int32_t)m->n_real);
     TileTables T{};
-    T.ntiles = (m->n_real + kTile - 1) / kTile;
+    T.ntiles = (int64_t)start.size() - 1;
     const int64_t nt = T.ntiles, ns = nt * kSlices;
-    if (nt == 0) return FDU_OK;
-    const TileSource S{m->n_real, m->slice_voff, m->slice_eoff, m->svid, m->seid, m->swf32, m->swg32, m->swe32};
+    fdu_status st;
+    int32_t *dstart = nullptr;
+    if ((st = m->upload(dstart, start))) return st;
+    const TileSource S{dstart, m->slice_voff, m->slice_eoff, m->svid, m->seid, m->swf32, m->swg32, m->swe32};
     // one allocation: the positions' order, the offsets (nt + 1, nt + 1, ns + 1, ns + 1)
     const int64_t noff = 2 * (nt + 1) + 2 * (ns + 1);
     int32_t *base = nullptr;
-    fdu_status st;
     if ((st = m->alloc(base, nt * kTile + noff))) return st;
     T.perm = base;
     T.voff = base + nt * kTile;
@@ -942,7 +954,7 @@ cudaError_t enqueue_step_persistent(fdu_mesh *m, int prec, cudaStream_t s, unsig
         a.comp = m->comp;
         a.dt_comp = m->dt_comp;
         cudaError_t e = launch_stage_persistent(prec, stage, ea, a, m->bar, m->bar + 1, expected, spin_limit,
-                                                m->bar_err, m->pl_threads, m->pl_blocks, s);
+                                                m->bar_err, m->pl_threads, m->pl_blocks, m->tile32, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1452,7 +1464,7 @@ fdu_status fdu_batch_create(int32_t n_meshes, const double *const *xy, const int
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
         m->pl_threads = 256;
-        m->pl_blocks = sms * std::max(1, persistent_blocks_per_sm(32, 256, false));
+        m->pl_blocks = sms * std::max(1, persistent_blocks_per_sm(32, 256, false, m->tile32));
         if (cudaGetLastError() != cudaSuccess) st = set_err(FDU_ERR_CUDA, "batch setup");
     }
     if (st != FDU_OK) {
@@ -1518,7 +1530,7 @@ fdu_status fdu_batch_set_launch(fdu_mesh *m, int threads, int blocks_per_sm) {
     if (threads != 128 && threads != 256 && threads != 512) return set_err(FDU_ERR_ARG, "threads must be 128, 256, 512");
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-    const int occ = std::max(persistent_blocks_per_sm(64, threads, m->dw64), persistent_blocks_per_sm(32, threads, false));
+    const int occ = std::max(persistent_blocks_per_sm(64, threads, m->dw64, m->tile32), persistent_blocks_per_sm(32, threads, false, m->tile32));
     if (blocks_per_sm < 1 || blocks_per_sm > occ)
         return set_err(FDU_ERR_ARG, "blocks_per_sm must be 1.." + std::to_string(occ) + " at " +
                                         std::to_string(threads) + " threads");
@@ -1549,7 +1561,7 @@ fdu_status fdu_batch_rk_steps(fdu_mesh *m, int precision, int n_steps, void *str
     if ((st = check_precision(m, precision))) return st;
     if (n_steps == 0) return FDU_OK;
     cudaStream_t s = m->stream(stream);
-    const int occ = persistent_blocks_per_sm(precision, m->pl_threads, m->dw64);
+    const int occ = persistent_blocks_per_sm(precision, m->pl_threads, m->dw64, m->tile32);
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
     if (occ < 1) return set_err(FDU_ERR_ARG, "the persistent kernel does not fit " + std::to_string(m->pl_threads) +
@@ -1599,7 +1611,7 @@ fdu_status fdu_batch_autotune(fdu_mesh *m, int precision, int *threads, int *blo
     double best = INFINITY;
     int bt = m->pl_threads, bb = m->pl_blocks / std::max(sms, 1);
     for (int t : {128, 256, 512}) {
-        const int occ = persistent_blocks_per_sm(precision, t, m->dw64);
+        const int occ = persistent_blocks_per_sm(precision, t, m->dw64, m->tile32);
         for (int k = 1; k <= occ; ++k) {
             m->pl_threads = t;
             m->pl_blocks = k * sms;
@@ -1658,9 +1670,9 @@ fdu_status fdu_batch_barrier_selftest(fdu_mesh *m, int *status) {
     a.dt_comp = m->dt_comp;
     int sms = 0;
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-    const int nb = std::min(m->pl_blocks, persistent_blocks_per_sm(32, m->pl_threads, false) * sms);
+    const int nb = std::min(m->pl_blocks, persistent_blocks_per_sm(32, m->pl_threads, false, m->tile32) * sms);
     CK(launch_stage_persistent(32, 1, ea, a, m->bar, m->bar + 1, (unsigned)nb + 1, 20000, m->bar_err, m->pl_threads,
-                               nb, s));
+                               nb, m->tile32, s));
     // an ordinary step enqueued behind the failed launch, before the error is
     // read: each of its launches finds the flag set and returns at entry (it
     // neither arrives on the count the failed barrier left nor writes the state)

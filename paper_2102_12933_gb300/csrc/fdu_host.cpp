@@ -781,19 +781,29 @@ int build_host_tables(const double *xy, int64_t nv, const CellList &cells, int a
     T.v_new2old.resize(nv);
     std::iota(T.v_new2old.begin(), T.v_new2old.end(), 0);
     if (o.renumber) {
-        double lo[2] = {INFINITY, INFINITY}, hi[2] = {-INFINITY, -INFINITY};
-        for (int64_t v = 0; v < nv; ++v)
-            for (int c = 0; c < 2; ++c) {
-                lo[c] = std::min(lo[c], T.xy[2 * v + c]);
-                hi[c] = std::max(hi[c], T.xy[2 * v + c]);
-            }
+        // each mesh of a batch is ordered inside its own bounding box, so that its
+        // vertices and edges come in the order they have in the mesh alone
+        struct Box {
+            double lo[2] = {INFINITY, INFINITY}, hi[2] = {-INFINITY, -INFINITY}, scale = 0;
+        };
         const int order = 16;
-        const double span = std::max(hi[0] - lo[0], hi[1] - lo[1]);
-        const double scale = span > 0 ? ((1 << order) - 1) / span : 0;
+        std::vector<Box> box(comp ? 1 + *std::max_element(comp, comp + nv) : 1);
+        for (int64_t v = 0; v < nv; ++v) {
+            Box &b = box[comp ? comp[v] : 0];
+            for (int c = 0; c < 2; ++c) {
+                b.lo[c] = std::min(b.lo[c], T.xy[2 * v + c]);
+                b.hi[c] = std::max(b.hi[c], T.xy[2 * v + c]);
+            }
+        }
+        for (Box &b : box) {
+            const double span = std::max(b.hi[0] - b.lo[0], b.hi[1] - b.lo[1]);
+            b.scale = span > 0 ? ((1 << order) - 1) / span : 0;
+        }
         std::vector<uint64_t> key(nv);
         for (int64_t v = 0; v < nv; ++v) {
-            uint32_t ix = (uint32_t)((T.xy[2 * v] - lo[0]) * scale);
-            uint32_t iy = (uint32_t)((T.xy[2 * v + 1] - lo[1]) * scale);
+            const Box &b = box[comp ? comp[v] : 0];
+            const uint32_t ix = (uint32_t)((T.xy[2 * v] - b.lo[0]) * b.scale);
+            const uint32_t iy = (uint32_t)((T.xy[2 * v + 1] - b.lo[1]) * b.scale);
             key[v] = hilbert_index(ix, iy, order);
         }
         std::stable_sort(T.v_new2old.begin(), T.v_new2old.end(),

@@ -896,8 +896,8 @@ __global__ void __launch_bounds__(kTileThreads)
     extern __shared__ int tile_work[];
     TileWork &W = *reinterpret_cast<TileWork *>(tile_work);
     __shared__ int key[kTile];
-    const int64_t t = blockIdx.x, v0 = t * kTile;
-    const int nvt = (int)min((int64_t)kTile, S.n_real - v0), i = threadIdx.x;
+    const int64_t t = blockIdx.x, p0 = t * kTile, v0 = S.start[t];
+    const int nvt = S.start[t + 1] - S.start[t], i = threadIdx.x;
     TileRow r{0, 0, 0, 0};
     if (i < kTile) {
         if (i < nvt) r = tile_row(S, v0 + i);
@@ -909,7 +909,7 @@ __global__ void __launch_bounds__(kTileThreads)
         for (int q = 0; q < kTile; ++q) rank += key[q] > key[i] || (key[q] == key[i] && q < i);
         W.J[rank] = r.J;
         W.K[rank] = r.K;
-        T.perm[v0 + rank] = i < nvt ? (int32_t)(v0 + i) : -1;
+        T.perm[p0 + rank] = i < nvt ? (int32_t)(v0 + i) : -1;
     }
     __syncthreads();
     if (i < kTile / kSell) {
@@ -975,9 +975,9 @@ __device__ void tile_schedule(TileWork &W, int group, int steps, const int *n) {
 __global__ void __launch_bounds__(kTileThreads) tile_fill_kernel(TileSource S, TileTables T) {
     extern __shared__ int tile_work[];
     TileWork &W = *reinterpret_cast<TileWork *>(tile_work);
-    const int64_t t = blockIdx.x, v0 = t * kTile;
-    const int nvt = (int)min((int64_t)kTile, S.n_real - v0), i = threadIdx.x;
-    const int32_t v = i < kTile ? T.perm[v0 + i] : -1;
+    const int64_t t = blockIdx.x, p0 = t * kTile, v0 = S.start[t];
+    const int nvt = S.start[t + 1] - S.start[t], i = threadIdx.x;
+    const int32_t v = i < kTile ? T.perm[p0 + i] : -1;
     const TileRow r = v >= 0 ? tile_row(S, v) : TileRow{0, 0, 0, 0};
     const int64_t sl = t * (kTile / kSell) + i / kSell, lane = i % kSell;
     for (int part = 0; part < 2; ++part) {
@@ -1068,30 +1068,30 @@ __device__ __forceinline__ float4 ld_stream(const float4 *p) {
 // registers and 7 blocks per SM instead of 64 and 8 0.0417.  Tiles of 256
 // (0.054), table groups read ahead explicitly (0.044 to 0.064) and 6 or 9
 // blocks per SM (0.052, 0.045) are slower.
-template <int MODE>
-__global__ void __launch_bounds__(kTile, 7) div_f32_tile_kernel(const __grid_constant__ DivArgs A,
-                                                                 const __grid_constant__ TileTables T) {
-    extern __shared__ float4 sm[];
-    if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;
-    const int64_t t = blockIdx.x;
+//
+// One tile by kTile threads (tid of them, staging in sm); sync() holds those
+// threads until the staging of all is done.
+template <int MODE, class Sync>
+__device__ __forceinline__ void div_f32_tile_body(const DivArgs &A, const TileTables &T, const int64_t t, const int tid,
+                                                  float4 *sm, Sync &&sync) {
     const int v0 = __ldg(T.voff + t), nvt = __ldg(T.voff + t + 1) - v0;
     const int e0 = __ldg(T.eoff + t), net = __ldg(T.eoff + t + 1) - e0;
     float4 *sf = sm, *sg = sm + nvt, *sr = sm + 2 * nvt;
     const float4 *__restrict__ F = static_cast<const float4 *>(A.F);
     const float4 *__restrict__ r = static_cast<const float4 *>(A.r);
-    for (int i = threadIdx.x; i < net; i += kTile) cp_async16(sr + i, r + __ldg(T.elist + e0 + i));
-    for (int i = threadIdx.x; i < nvt; i += kTile) {
+    for (int i = tid; i < net; i += kTile) cp_async16(sr + i, r + __ldg(T.elist + e0 + i));
+    for (int i = tid; i < nvt; i += kTile) {
         const int64_t j = __ldg(T.vlist + v0 + i);
         cp_async16(sf + i, F + 2 * j);
         cp_async16(sg + i, F + 2 * j + 1);
     }
-    const int64_t sl = t * (kTile / kSell) + threadIdx.x / kSell;
-    const int lane = threadIdx.x % kSell;
-    const int32_t v = __ldg(T.perm + t * kTile + threadIdx.x);
+    const int64_t sl = t * (kTile / kSell) + tid / kSell;
+    const int lane = tid % kSell;
+    const int32_t v = __ldg(T.perm + t * kTile + tid);
     const int gb = __ldg(T.gvoff + sl), ge = __ldg(T.gvoff + sl + 1);
     const int hb = __ldg(T.geoff + sl), he = __ldg(T.geoff + sl + 1);
     cp_async_wait();
-    __syncthreads();
+    sync();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     auto vert = [&](int j, float a, float c) {
         const float4 f = sf[j], g = sg[j];
@@ -1126,6 +1126,13 @@ __global__ void __launch_bounds__(kTile, 7) div_f32_tile_kernel(const __grid_con
         edge(k.w, a.w);
     }
     if (v >= 0) div_f32_finish<MODE>(A, v, acc);
+}
+template <int MODE>
+__global__ void __launch_bounds__(kTile, 7) div_f32_tile_kernel(const __grid_constant__ DivArgs A,
+                                                                 const __grid_constant__ TileTables T) {
+    extern __shared__ float4 sm[];
+    if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;
+    div_f32_tile_body<MODE>(A, T, blockIdx.x, threadIdx.x, sm, [] { __syncthreads(); });
 }
 
 // Folded tables of the double-word divergence (launch_fold_tables); thread i
@@ -1241,10 +1248,14 @@ __device__ __forceinline__ bool barrier_failed(const int *err) {
 
 // One SSP-RK3 stage over every mesh of a batch in one cooperative launch:
 // all edge fluxes, a grid barrier, then every vertex's divergence and stage
-// update (grid-stride loops; MODE = stage 1..3).
-template <int PREC, int MODE>
-__global__ void stage_persistent_kernel(EdgeArgs EA, DivArgs DA, unsigned int *bar_count, unsigned int *bar_gen,
-                                        unsigned int nblocks_expected, unsigned long long spin_limit, int *err) {
+// update (grid-stride loops; MODE = stage 1..3).  TILES (FP32): each kTile
+// threads of a block take divergence tiles of their own, with T.smem bytes of
+// the dynamic shared memory and a named barrier (1 .. blockDim / kTile).
+template <int PREC, int MODE, bool TILES>
+__global__ void stage_persistent_kernel(const __grid_constant__ EdgeArgs EA, const __grid_constant__ DivArgs DA,
+                                        unsigned int *bar_count, unsigned int *bar_gen, unsigned int nblocks_expected,
+                                        unsigned long long spin_limit, int *err,
+                                        const __grid_constant__ TileTables T) {
     if (barrier_failed(err)) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1255,6 +1266,26 @@ __global__ void stage_persistent_kernel(EdgeArgs EA, DivArgs DA, unsigned int *b
     }
     __threadfence();
     if (!grid_barrier(bar_count, bar_gen, nblocks_expected, spin_limit, err)) return;
+    if (TILES) {
+        extern __shared__ float4 tile_stage[];
+        const int group = (int)threadIdx.x / kTile, groups = (int)blockDim.x / kTile;
+        float4 *sm = tile_stage + (int64_t)group * (T.smem / (int)sizeof(float4));
+        // barrier numbers as constants: a register operand would reserve all 16 of
+        // a block, and the SM's 64 then hold four blocks
+        const auto sync = [group] {
+            switch (group) {
+                case 0: asm volatile("bar.sync 1, %0;" ::"n"(kTile) : "memory"); break;
+                case 1: asm volatile("bar.sync 2, %0;" ::"n"(kTile) : "memory"); break;
+                case 2: asm volatile("bar.sync 3, %0;" ::"n"(kTile) : "memory"); break;
+                default: asm volatile("bar.sync 4, %0;" ::"n"(kTile) : "memory"); break;
+            }
+        };
+        for (int64_t t = (int64_t)blockIdx.x * groups + group; t < T.ntiles; t += (int64_t)gridDim.x * groups) {
+            div_f32_tile_body<MODE>(DA, T, t, (int)threadIdx.x % kTile, sm, sync);
+            sync();  // the next tile's staging takes the same memory
+        }
+        return;
+    }
     for (int64_t v = t0; v < DA.n_real; v += stride) {
         if (PREC == 64) div_f64_body<MODE>(DA, v);
         else div_f32_body<MODE>(DA, v);
@@ -1494,14 +1525,36 @@ void launch_max_dt(const double *w, const double *hmin, int64_t n, double gamma,
 }
 
 namespace {
-template <int PREC, int MODE>
-cudaError_t coop(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigned int *g, unsigned int ne,
-                 unsigned long long lim, int *err, int threads, int nb, cudaStream_t s) {
+// Dynamic shared memory of the FP32 persistent stage, 0 where it does without
+// tiles: kTileGroups groups of kTile threads have to fit an SM, as many as the
+// kernel's registers allow, so that every launch shape that fits without the
+// staging fits with it.
+constexpr int kTileGroups = 6;
+size_t persistent_tile_bytes(const TileTables &t, int threads) {
+    const size_t bytes = (size_t)t.smem * (threads / kTile);
+    return t.smem > 0 && (size_t)t.smem * kTileGroups <= (size_t)220 * 1024 ? bytes : 0;
+}
+template <int PREC, int MODE, bool TILES>
+cudaError_t coop_t(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigned int *g, unsigned int ne,
+                   unsigned long long lim, int *err, int threads, int nb, const TileTables &tt, size_t bytes,
+                   cudaStream_t s) {
     EdgeArgs a = ea;
     DivArgs d = da;
-    void *args[] = {&a, &d, &c, &g, &ne, &lim, &err};
-    return cudaLaunchCooperativeKernel((const void *)stage_persistent_kernel<PREC, MODE>, dim3(nb), dim3(threads),
-                                       args, 0, s);
+    TileTables t = tt;
+    void *args[] = {&a, &d, &c, &g, &ne, &lim, &err, &t};
+    const void *k = (const void *)stage_persistent_kernel<PREC, MODE, TILES>;
+    if (bytes > 0) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaLaunchCooperativeKernel(k, dim3(nb), dim3(threads), args, bytes, s);
+}
+template <int PREC, int MODE>
+cudaError_t coop(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsigned int *g, unsigned int ne,
+                 unsigned long long lim, int *err, int threads, int nb, const TileTables &t, cudaStream_t s) {
+    const size_t bytes = PREC == 32 ? persistent_tile_bytes(t, threads) : 0;
+    if (bytes > 0) return coop_t<PREC, MODE, PREC == 32>(ea, da, c, g, ne, lim, err, threads, nb, t, bytes, s);
+    return coop_t<PREC, MODE, false>(ea, da, c, g, ne, lim, err, threads, nb, t, 0, s);
 }
 }  // namespace
 
@@ -1524,7 +1577,8 @@ cudaError_t coop48(const EdgeArgs &ea, const DivArgs &da, unsigned int *c, unsig
 
 cudaError_t launch_stage_persistent(int prec, int mode, const EdgeArgs &ea, const DivArgs &da, unsigned int *bar_count,
                                     unsigned int *bar_gen, unsigned int nblocks_expected,
-                                    unsigned long long spin_limit, int *err, int threads, int nb, cudaStream_t s) {
+                                    unsigned long long spin_limit, int *err, int threads, int nb, const TileTables &t,
+                                    cudaStream_t s) {
     const unsigned int ne = nblocks_expected;
     if (prec == 48) {
         if (mode == 1) return coop48<1, false>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
@@ -1537,13 +1591,13 @@ cudaError_t launch_stage_persistent(int prec, int mode, const EdgeArgs &ea, cons
         return coop48<3, true>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
     }
     if (prec == 64) {
-        if (mode == 1) return coop<64, 1>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
-        if (mode == 2) return coop<64, 2>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
-        return coop<64, 3>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+        if (mode == 1) return coop<64, 1>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, t, s);
+        if (mode == 2) return coop<64, 2>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, t, s);
+        return coop<64, 3>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, t, s);
     }
-    if (mode == 1) return coop<32, 1>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
-    if (mode == 2) return coop<32, 2>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
-    return coop<32, 3>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, s);
+    if (mode == 1) return coop<32, 1>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, t, s);
+    if (mode == 2) return coop<32, 2>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, t, s);
+    return coop<32, 3>(ea, da, bar_count, bar_gen, ne, spin_limit, err, threads, nb, t, s);
 }
 
 namespace {
@@ -1560,16 +1614,26 @@ int dw_blocks_per_sm(int threads) {
 }
 }  // namespace
 
-int persistent_blocks_per_sm(int prec, int threads, bool guard) {
+int persistent_blocks_per_sm(int prec, int threads, bool guard, const TileTables &t) {
     int n = 0;
     // the three stage modes share their register footprint; mode 3 stands for all
     if (prec == 48) return dw_blocks_per_sm<false>(threads);
     if (prec == 64) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<64, 3>, threads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<64, 3, false>, threads, 0);
         // a block the FP64 kernel has no registers for is refused at precision 64 on either path
         return guard && n > 0 ? dw_blocks_per_sm<true>(threads) : n;
     }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<32, 3>, threads, 0);
+    const size_t bytes = persistent_tile_bytes(t, threads);
+    if (bytes > 0) {
+        for (auto k : {stage_persistent_kernel<32, 1, true>, stage_persistent_kernel<32, 2, true>,
+                       stage_persistent_kernel<32, 3, true>})
+            if (cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) !=
+                cudaSuccess)
+                return 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<32, 3, true>, threads, bytes);
+    } else {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stage_persistent_kernel<32, 3, false>, threads, 0);
+    }
     return n;
 }
 

@@ -99,7 +99,9 @@ struct DivArgs {
     unsigned long long *limited; // vertices whose stage update the safeguard scaled
 };
 
-// ---- Divergence tiles.  A tile is kTile consecutive vertices (internal order).
+// ---- Divergence tiles.  A tile is up to kTile consecutive vertices (internal
+// order) of one mesh: a batch starts a tile at each of its meshes, so that a
+// vertex's entries are summed in the order they have in the mesh alone.
 // The distinct vertices and edges of its stencils are listed once (ascending
 // ids), a block copies their fluxes into shared memory, and the stencil entries
 // name them by 16-bit position in those lists.  Inside a tile the vertices are
@@ -110,7 +112,7 @@ constexpr int kTile = 128;
 constexpr int kTileMaxV = 1024, kTileMaxE = 2048;  // capacity of a tile's lists
 // Source of the tiles: a SELL layout of the divergence tables.
 struct TileSource {
-    int64_t n_real;
+    const int32_t *start;  // [ntiles + 1] first vertex of each tile
     const int64_t *slice_voff, *slice_eoff;
     const int32_t *vid, *eid;
     const float *wf, *wg, *we;
@@ -182,9 +184,11 @@ void launch_max_dt(const double *w, const double *hmin, int64_t n, double gamma,
 // normal use) and gives up after `spin_limit` polls, setting *err.
 cudaError_t launch_stage_persistent(int prec, int mode, const EdgeArgs &ea, const DivArgs &da, unsigned int *bar_count,
                                     unsigned int *bar_gen, unsigned int nblocks_expected,
-                                    unsigned long long spin_limit, int *err, int threads, int blocks, cudaStream_t s);
+                                    unsigned long long spin_limit, int *err, int threads, int blocks,
+                                    const TileTables &tiles, cudaStream_t s);
 // Co-resident blocks per SM of the persistent stage kernel at `threads`; guard:
-// the mesh's precision-64 kernel takes the double-word path (kDivGuard).
-int persistent_blocks_per_sm(int prec, int threads, bool guard);
+// the mesh's precision-64 kernel takes the double-word path (kDivGuard); tiles:
+// its FP32 divergence tiles.
+int persistent_blocks_per_sm(int prec, int threads, bool guard, const TileTables &tiles);
 
 }  // namespace fdu
