@@ -87,7 +87,7 @@ struct fdu_mesh {
     float4 *w32 = nullptr;                                  // [nv]
     double *r64 = nullptr;                                  // [ne_act][4]
     float4 *r32 = nullptr;                                  // [ne_act]
-    unsigned long long *counters = nullptr;  // [0] fallbacks, [1] dt slot, [2] adaptive slot, [3] unused,
+    unsigned long long *counters = nullptr;  // [0] fallbacks, [1] dt slot, [2] adaptive slot, [3] blocks of a reduction done,
                                              // [4] stage updates scaled by the positivity safeguard,
                                              // [5] first non-physical row of a state being set
     // adaptive stepping: (t, dt, nonphysical flag), then the step counter and
@@ -672,9 +672,8 @@ void enqueue_stages(fdu_mesh *m, int prec, double dt, const double *dt_dev, cuda
         if (m->n_ghost > 0) {
             // Dirichlet ghosts take their fixed values from the step's start buffers (wn, F[0], Q[0])
             const void *F0 = f64 ? (const void *)m->F64[0] : (const void *)m->F32[0];
-            launch_ghost_fill(a.wout, m->wn, a.Fout, F0, fq, prec == 32 ? m->w32 : nullptr, m->donor, m->n_real,
-                              m->n_ghost, s);
-            if (a.Qout) launch_ghost_fill(nullptr, nullptr, a.Qout, m->Q64[0], 2, nullptr, m->donor, m->n_real, m->n_ghost, s);
+            launch_ghost_fill(a.wout, m->wn, a.Fout, F0, fq, a.Qout, m->Q64[0], prec == 32 ? m->w32 : nullptr, m->donor,
+                              m->n_real, m->n_ghost, s);
         }
     }
 }
@@ -964,8 +963,8 @@ cudaError_t enqueue_step_persistent(fdu_mesh *m, int prec, cudaStream_t s, unsig
 // dt = min(cfl * bound, t_end - t) into tstate, then the three stages read
 // dt from there (and skip their work once t_end is reached).
 void enqueue_adaptive_step(fdu_mesh *m, int prec, double cfl, double t_end, cudaStream_t s) {
-    launch_max_dt(m->wn, m->hmin, m->n_real, m->opts.gamma, m->counters + 2, s);
-    launch_dt_finalize(m->counters + 2, m->tstate, cfl, t_end, m->nsteps, s);
+    launch_max_dt(m->wn, m->hmin, m->n_real, m->opts.gamma, m->counters + 2, s, nullptr,
+                  DtFinal{m->tstate, cfl, t_end, m->nsteps, reinterpret_cast<unsigned int *>(m->counters + 3)});
     enqueue_step(m, prec, 0.0, m->tstate + 1, s, false);
 }
 
@@ -1188,7 +1187,8 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
         CK_LAUNCH();
     }
     if (m->n_ghost > 0) {
-        launch_ghost_fill(m->wn, nullptr, nullptr, nullptr, 0, nullptr, m->donor, m->n_real, m->n_ghost, s);
+        launch_ghost_fill(m->wn, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, m->donor, m->n_real,
+                                         m->n_ghost, s);
         CK_LAUNCH();
     }
     m->f64_valid = m->f32_valid = false;
@@ -1708,7 +1708,8 @@ fdu_status fdu_residual_noalloc(const fdu_mesh *mc, const double *w, double *dwd
     // ghost rows of the output must start at zero
     if (m->n_ghost > 0) CK(cudaMemsetAsync(dwdt, 0, 4 * m->nv * sizeof(double), s));
     launch_permute_rows(w, wi, m->new2old, m->nv, true, s);
-    if (m->n_ghost > 0) launch_ghost_fill(wi, nullptr, nullptr, nullptr, 0, nullptr, m->donor, m->n_real, m->n_ghost, s);
+    if (m->n_ghost > 0) launch_ghost_fill(wi, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr, m->donor, m->n_real,
+                                         m->n_ghost, s);
     launch_vertex_flux_f64(wi, F, m->nv, m->opts.gamma, s);
     EdgeArgs ea = edge_args(m, 64, wi);
     ea.r = r;

@@ -252,11 +252,14 @@ template <int MODE> __device__ __forceinline__ float2 tld(const float2 *p) {
     asm("ld.global.nc.L1::no_allocate.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
 }
-template <int MODE, bool DWE = false>
-__device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) {
-    const int64_t sl = i / kSell;
-    const int lane = (int)(i % kSell);
-    const int64_t v = A.perm ? (int64_t)__ldg(A.perm + i) : i;
+// With LPV > 1 that many consecutive lanes share a position: lane q of them
+// takes every LPV-th entry, the partial sums meet by shuffles (every lane of the
+// warp calls it, `on` where its position exists) and lane 0 goes on.
+template <int MODE, bool DWE = false, int LPV = 1>
+__device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i, const int q = 0, const bool on = true) {
+    const int64_t sl = on ? i / kSell : 0;
+    const int lane = (int)(i % kSell) + q * kSell;
+    const int64_t v = !on ? 0 : A.perm ? (int64_t)__ldg(A.perm + i) : i;
     const double *__restrict__ F = static_cast<const double *>(A.F);
     const double *__restrict__ r = static_cast<const double *>(A.r);
     const double *__restrict__ wf = DWE ? A.wf48 : static_cast<const double *>(A.wf);
@@ -264,9 +267,9 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
     const double *__restrict__ we = static_cast<const double *>(A.we);
     dbl4 acc = dbl4_make(0, 0, 0, 0);
     {
-        const int64_t b = __ldg(A.slice_voff + sl) + lane, e = __ldg(A.slice_voff + sl + 1);
+        const int64_t b = __ldg(A.slice_voff + sl) + lane, e = on ? __ldg(A.slice_voff + sl + 1) : 0;
 #pragma unroll 4
-        for (int64_t p = b; p < e; p += kSell) {
+        for (int64_t p = b; p < e; p += LPV * kSell) {
             const int32_t j = tld<MODE>(A.vid + p);
             const double a = tld<MODE>(wf + p), c = tld<MODE>(wg + p);
             const dbl4 f = ld4v(F, 2 * (int64_t)j), g = ld4v(F, 2 * (int64_t)j + 1);
@@ -281,9 +284,9 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
         const float2 *__restrict__ we2 = A.we48;
         const float4 *__restrict__ rd = static_cast<const float4 *>(A.r);
         dot2 sx{0.0f, 0.0f}, sy = sx, sz = sx, sw = sx;
-        const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = __ldg(A.slice_eoff + sl + 1);
+        const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = on ? __ldg(A.slice_eoff + sl + 1) : 0;
 #pragma unroll 6
-        for (int64_t p = b; p < e; p += kSell) {
+        for (int64_t p = b; p < e; p += LPV * kSell) {
             const int32_t k = tld<MODE>(A.eid + p);
             const float2 wq = tld<MODE>(we2 + p);
             const dw a = dw_make(wq.x, wq.y);
@@ -300,17 +303,27 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
         acc.z += f2d(rz.h) + f2d(rz.l);
         acc.w += f2d(rw.h) + f2d(rw.l);
     } else {
-        const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = __ldg(A.slice_eoff + sl + 1);
+        const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = on ? __ldg(A.slice_eoff + sl + 1) : 0;
 #pragma unroll 4
-        for (int64_t p = b; p < e; p += kSell) {
+        for (int64_t p = b; p < e; p += LPV * kSell) {
             const int32_t k = tld<MODE>(A.eid + p);
             const double a = tld<MODE>(we + p);
-            const dbl4 q = ld4v(r, k);
-            acc.x = fma(a, q.x, acc.x);
-            acc.y = fma(a, q.y, acc.y);
-            acc.z = fma(a, q.z, acc.z);
-            acc.w = fma(a, q.w, acc.w);
+            const dbl4 s = ld4v(r, k);
+            acc.x = fma(a, s.x, acc.x);
+            acc.y = fma(a, s.y, acc.y);
+            acc.z = fma(a, s.z, acc.z);
+            acc.w = fma(a, s.w, acc.w);
         }
+    }
+    if (LPV > 1) {
+#pragma unroll
+        for (int o = 1; o < LPV; o <<= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+            acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+        }
+        if (q != 0 || !on) return;
     }
     {
         const double *cfg = DWE ? A.cfg48 : static_cast<const double *>(A.cfg);
@@ -356,11 +369,16 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i) 
 template <int MODE>
 __device__ __noinline__ void div_f64_cold(const DivArgs *A, const int64_t i) { div_f64_body<MODE, false>(*A, i); }
 // The divergence of one vertex by KIND (kDivPlain, kDivDw, kDivGuard).
-template <int MODE, int KIND>
-__device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, const bool wide) {
-    if (KIND == kDivPlain) div_f64_body<MODE, false>(A, i);
-    else if (KIND == kDivGuard && wide) div_f64_cold<MODE>(&A, i);
-    else div_f64_body<MODE, true>(A, i);
+template <int MODE, int KIND, int LPV = 1>
+__device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, const bool wide, const int q = 0,
+                                            const bool on = true) {
+    if (KIND == kDivPlain) {
+        div_f64_body<MODE, false, LPV>(A, i, q, on);
+    } else if (KIND == kDivGuard && wide) {
+        if (q == 0 && on) div_f64_cold<MODE>(&A, i);
+    } else {
+        div_f64_body<MODE, true, LPV>(A, i, q, on);
+    }
 }
 
 // ================================================================== FP32 path
@@ -785,12 +803,13 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) edge_flux_guard_kernel(const __
 // At most 80 registers (6 blocks, 24 warps per SM): with the 56 the compiler
 // takes when left alone fewer gathers are in flight (precision 48 0.139 against
 // 0.120 ms at 250k vertices; 64 registers 0.123, 40 with 9 blocks 0.139).
-template <int MODE, int KIND>
+template <int MODE, int KIND, int LPV>
 __global__ void __launch_bounds__(kDivBlock, 6) div_f64_kernel(const __grid_constant__ DivArgs A) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= A.n_real) return;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LPV;
+    if (LPV == 1 && i >= A.n_real) return;
     if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;  // adaptive run already at t_end
-    div_f64_any<MODE, KIND>(A, v, KIND == kDivGuard && stage_is_wide(A.wide, A.wide_in));
+    div_f64_any<MODE, KIND, LPV>(A, i, KIND == kDivGuard && stage_is_wide(A.wide, A.wide_in),
+                                 (int)threadIdx.x % LPV, i < A.n_real);
 }
 // ------------------------------------------------------------------ divergence tiles
 constexpr int kTileThreads = 256;  // threads of the tile-building kernels
@@ -1341,9 +1360,11 @@ __global__ void permute_rows_kernel(const double *__restrict__ in, double *__res
 // state and fluxes from wsrc / Fsrc, the buffers of the step's start state
 // (a no-op when they are the buffers being filled).  F holds `fq` 16-byte
 // words per vertex.
+// (F, Fsrc) and (Q, Qsrc): vertex fluxes and, for an FP64 state, Roe records
+// (2 words per vertex), in the one launch.
 __global__ void ghost_fill_kernel(double *__restrict__ w, const double *wsrc, uint4 *__restrict__ F, const uint4 *Fsrc,
-                                  int fq, float4 *__restrict__ w32, const int32_t *__restrict__ donor, int64_t n_real,
-                                  int64_t n_ghost) {
+                                  int fq, uint4 *__restrict__ Q, const uint4 *Qsrc, float4 *__restrict__ w32,
+                                  const int32_t *__restrict__ donor, int64_t n_real, int64_t n_ghost) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_ghost) return;
     const int64_t g = n_real + i, d = __ldg(donor + i);
@@ -1351,34 +1372,110 @@ __global__ void ghost_fill_kernel(double *__restrict__ w, const double *wsrc, ui
         if (w && wsrc && w != wsrc) st4(w, g, ld4(wsrc, g));
         if (F && Fsrc && F != Fsrc)
             for (int c = 0; c < fq; ++c) F[fq * g + c] = Fsrc[fq * g + c];
+        if (Q && Qsrc && Q != Qsrc)
+            for (int c = 0; c < 2; ++c) Q[2 * g + c] = Qsrc[2 * g + c];
         return;
     }
     if (w) st4(w, g, ld4(w, d));
     if (F)
         for (int c = 0; c < fq; ++c) F[fq * g + c] = F[fq * d + c];
+    if (Q)
+        for (int c = 0; c < 2; ++c) Q[2 * g + c] = Q[2 * d + c];
     if (w32) w32[g] = w32[d];
 }
 
-// min over vertices of h_v / (|u| + c), as the bit pattern of a positive double
-__global__ void max_dt_kernel(const double *__restrict__ w, const double *__restrict__ hmin, int64_t n, double gamma,
-                              unsigned long long *slot, const int32_t *__restrict__ comp) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double t = INFINITY;
-    if (v < n) {
-        const dbl4 s = ld4(w, v);
-        const double ir = 1.0 / s.x;
-        const double u = s.y * ir, vv = s.z * ir;
-        const double p = (gamma - 1.0) * (s.w - 0.5 * (s.y * u + s.z * vv));
-        const double c = sqrt(gamma * p * ir);
-        t = hmin[v] / (sqrt(u * u + vv * vv) + c);
-        if (!(t > 0)) t = 0;  // non-physical state: report dt = 0
+// h / (|u| + c) of a state (0 where it is non-physical)
+__device__ __forceinline__ double dt_bound64(const dbl4 &s, double h, double gamma) {
+    const double ir = 1.0 / s.x;
+    const double u = s.y * ir, v = s.z * ir;
+    const double p = (gamma - 1.0) * (s.w - 0.5 * (s.y * u + s.z * v));
+    const double c = sqrt(gamma * p * ir);
+    const double t = h / (sqrt(u * u + v * v) + c);
+    return t > 0 ? t : 0.0;
+}
+// Adaptive step from the reduced bound in *slot; runs in one thread once every
+// vertex has been reduced.  tstate = (t, dt, nonphysical); the slot is reset.
+__device__ __forceinline__ void dt_finalize(unsigned long long *slot, double *tstate, double cfl, double t_end,
+                                            unsigned long long *nsteps) {
+    const double bound = __longlong_as_double((long long)*(volatile unsigned long long *)slot);
+    const double t = tstate[0];
+    double dt = cfl * bound;
+    const double rem = t_end - t;
+    if (!(bound > 0.0) || !(bound < INFINITY)) {
+        dt = 0.0;
+        tstate[2] = 1.0;  // non-physical state
+    } else if (rem <= 1e-12 * fabs(t_end)) {
+        dt = 0.0;
+    } else if (rem < dt) {
+        dt = rem;
     }
+    tstate[1] = dt;
+    tstate[0] = dt > 0.0 ? (rem < cfl * bound ? t_end : t + dt) : t;
+    if (dt > 0.0) *nsteps += 1;
+    *slot = 0x7FF0000000000000ull;
+}
+// min over vertices of h_v / (|u| + c), as the bit pattern of a positive double.
+// The FP64 divisions and square roots (about 65 instructions of 64 cycles a
+// warp) are taken only where the minimum can lie: the bound is estimated in
+// FP32, and a vertex whose estimate is above the block's smallest, or above the
+// minimum reduced so far, by more than 2^-10 is left out.  The estimate errs by
+// a few 2^-24 relative, times the Mach number through the pressure; a vertex
+// with p < 2^-10 rho E (Mach above 40), or outside FP32's comfortable range, is
+// always taken, so the result is the FP64 minimum itself.  With `fin` (adaptive stepping) the last block
+// also finalises the step.
+constexpr int kDtBlock = 256;
+__global__ void __launch_bounds__(kDtBlock)
+    max_dt_kernel(const double *__restrict__ w, const double *__restrict__ hmin, int64_t n, double gamma,
+                  unsigned long long *slot, const int32_t *__restrict__ comp, DtFinal fin) {
+    __shared__ float smallest[kDtBlock / 32];
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = v < n;
+    dbl4 s = dbl4_make(0, 0, 0, 0);
+    double h = 0.0;
+    float est = INFINITY;
+    bool sure = false;
+    if (on) {
+        s = ld4(w, v);
+        h = hmin[v];
+        const float g = (float)gamma, r = (float)s.x, mx = (float)s.y, my = (float)s.z, E = (float)s.w;
+        const float ir = 1.0f / r, ux = mx * ir, uy = my * ir;
+        const float p = (g - 1.0f) * (E - 0.5f * (mx * ux + my * uy));
+        const float speed = sqrtf(ux * ux + uy * uy) + sqrtf(g * p * ir);
+        est = (float)h / speed;
+        sure = !(p > 0x1p-10f * E && E > 0x1p-100f && speed > 0x1p-60f) || !(est > 0x1p-100f && est < INFINITY);
+    }
+    float m = sure ? INFINITY : est;
+    for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) smallest[threadIdx.x / 32] = m;
+    __syncthreads();
+    for (int i = 0; i < kDtBlock / 32; ++i) m = fminf(m, smallest[i]);
+    bool take = on && (sure || est <= m * (1.0f + 0x1p-10f));
     if (comp) {  // one slot per component
-        if (v < n) atomicMin(slot + __ldg(comp + v), (unsigned long long)__double_as_longlong(t));
+        // the block's smallest may belong to another component: compare with the component's own slot only
+        unsigned long long *own = slot + (on ? __ldg(comp + v) : 0);
+        const double so_far = __longlong_as_double((long long)__ldcg(own));
+        take = on && (sure || (double)est <= so_far * (1.0 + 0x1p-10));
+        if (take) atomicMin(own, (unsigned long long)__double_as_longlong(dt_bound64(s, h, gamma)));
         return;
     }
-    for (int o = 16; o > 0; o >>= 1) t = fmin(t, __shfl_xor_sync(0xffffffffu, t, o));
-    if ((threadIdx.x & 31) == 0) atomicMin(slot, (unsigned long long)__double_as_longlong(t));
+    if (take && !sure) {
+        const double so_far = __longlong_as_double((long long)__ldcg(slot));
+        take = (double)est <= so_far * (1.0 + 0x1p-10);
+    }
+    double t = INFINITY;
+    if (take) t = dt_bound64(s, h, gamma);
+    if (__any_sync(0xffffffffu, take)) {
+        for (int o = 16; o > 0; o >>= 1) t = fmin(t, __shfl_xor_sync(0xffffffffu, t, o));
+        if ((threadIdx.x & 31) == 0) atomicMin(slot, (unsigned long long)__double_as_longlong(t));
+    }
+    if (!fin.tstate) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(fin.done, 1u) == gridDim.x - 1) {
+        *fin.done = 0;
+        __threadfence();
+        dt_finalize(slot, fin.tstate, fin.cfl, fin.t_end, fin.nsteps);
+    }
 }
 
 // FMA-throughput probe: 8 independent chains x = x*a + b per thread.
@@ -1395,26 +1492,6 @@ __global__ void fma_probe_kernel(T *out, int iters, T a, T b) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) s += x[k];
     out[(int64_t)blockIdx.x * blockDim.x + threadIdx.x] = s;
-}
-
-__global__ void dt_finalize_kernel(unsigned long long *slot, double *tstate, double cfl, double t_end,
-                                   unsigned long long *nsteps) {
-    const double bound = __longlong_as_double((long long)*slot);
-    const double t = tstate[0];
-    double dt = cfl * bound;
-    const double rem = t_end - t;
-    if (!(bound > 0.0) || !(bound < INFINITY)) {
-        dt = 0.0;
-        tstate[2] = 1.0;  // non-physical state
-    } else if (rem <= 1e-12 * fabs(t_end)) {
-        dt = 0.0;
-    } else if (rem < dt) {
-        dt = rem;
-    }
-    tstate[1] = dt;
-    tstate[0] = dt > 0.0 ? (rem < cfl * bound ? t_end : t + dt) : t;
-    if (dt > 0.0) *nsteps += 1;
-    *slot = 0x7FF0000000000000ull;
 }
 
 // which: 0 recip64, 1 rsqrt64, 2 half64, 3 twice64
@@ -1463,21 +1540,33 @@ void launch_edge_flux_f32(const EdgeArgs &a, cudaStream_t s) {
     if (a.coef_gaps) edge_flux_f32_kernel<true><<<blocks(a.ne, kEdgeBlock), kEdgeBlock, 0, s>>>(a);
     else edge_flux_f32_kernel<false><<<blocks(a.ne, kEdgeBlock), kEdgeBlock, 0, s>>>(a);
 }
-template <int KIND>
+template <int KIND, int LPV>
 void launch_div_f64_t(const DivArgs &a, int mode, cudaStream_t s) {
-    const unsigned g = blocks(a.n_real, kDivBlock);
+    const unsigned g = blocks(a.n_real * LPV, kDivBlock);
     switch (mode) {
-        case 0: div_f64_kernel<0, KIND><<<g, kDivBlock, 0, s>>>(a); break;
-        case 1: div_f64_kernel<1, KIND><<<g, kDivBlock, 0, s>>>(a); break;
-        case 2: div_f64_kernel<2, KIND><<<g, kDivBlock, 0, s>>>(a); break;
-        default: div_f64_kernel<3, KIND><<<g, kDivBlock, 0, s>>>(a); break;
+        case 0: div_f64_kernel<0, KIND, LPV><<<g, kDivBlock, 0, s>>>(a); break;
+        case 1: div_f64_kernel<1, KIND, LPV><<<g, kDivBlock, 0, s>>>(a); break;
+        case 2: div_f64_kernel<2, KIND, LPV><<<g, kDivBlock, 0, s>>>(a); break;
+        default: div_f64_kernel<3, KIND, LPV><<<g, kDivBlock, 0, s>>>(a); break;
     }
+}
+template <int LPV>
+void launch_div_f64_l(const DivArgs &a, int mode, cudaStream_t s) {
+    if (a.kind == kDivGuard) launch_div_f64_t<kDivGuard, LPV>(a, mode, s);
+    else if (a.kind == kDivDw) launch_div_f64_t<kDivDw, LPV>(a, mode, s);
+    else launch_div_f64_t<kDivPlain, LPV>(a, mode, s);
 }
 void launch_div_f64(const DivArgs &a, int mode, cudaStream_t s) {
     if (a.n_real <= 0) return;
-    if (a.kind == kDivGuard) launch_div_f64_t<kDivGuard>(a, mode, s);
-    else if (a.kind == kDivDw) launch_div_f64_t<kDivDw>(a, mode, s);
-    else launch_div_f64_t<kDivPlain>(a, mode, s);
+    // Small meshes leave most of the chip's 152 x 24 resident warps empty while
+    // each thread walks 60 to 100 dependent gathers, so several lanes share a
+    // vertex.  RK3 step of the vortex at 1, 2, 4 lanes: 4096 vertices 84 / 68 / 56
+    // us, 10,000 94 / 82 / 79, 16,900 107 / 98 / 101, 48,400 195 / 183 / 214, 67,600
+    // 241 / 255 / 289 (the stage update is repeated by every warp, so more lanes
+    // cost FP64 time once the warps are there); 8 lanes win only below 2000.
+    if (a.n_real <= 12 * 1024) launch_div_f64_l<4>(a, mode, s);
+    else if (a.n_real <= 56 * 1024) launch_div_f64_l<2>(a, mode, s);
+    else launch_div_f64_l<1>(a, mode, s);
 }
 void launch_div_f32(const DivArgs &a, int mode, cudaStream_t s) {
     if (a.n_real <= 0) return;
@@ -1512,16 +1601,16 @@ void launch_check_rows(const double *w, int64_t n, unsigned long long *bad, cuda
 void launch_permute_rows(const double *in, double *out, const int32_t *map, int64_t n, bool gather, cudaStream_t s) {
     if (n > 0) permute_rows_kernel<<<blocks(n, 256), 256, 0, s>>>(in, out, map, n, gather);
 }
-void launch_ghost_fill(double *w, const double *wsrc, void *F, const void *Fsrc, int fq, float4 *w32,
-                       const int32_t *donor, int64_t n_real, int64_t n_ghost, cudaStream_t s) {
+void launch_ghost_fill(double *w, const double *wsrc, void *F, const void *Fsrc, int fq, double *Q, const double *Qsrc,
+                       float4 *w32, const int32_t *donor, int64_t n_real, int64_t n_ghost, cudaStream_t s) {
     if (n_ghost > 0)
-        ghost_fill_kernel<<<blocks(n_ghost, 256), 256, 0, s>>>(w, wsrc, static_cast<uint4 *>(F),
-                                                               static_cast<const uint4 *>(Fsrc), fq, w32, donor, n_real,
-                                                               n_ghost);
+        ghost_fill_kernel<<<blocks(n_ghost, 256), 256, 0, s>>>(
+            w, wsrc, static_cast<uint4 *>(F), static_cast<const uint4 *>(Fsrc), fq, reinterpret_cast<uint4 *>(Q),
+            reinterpret_cast<const uint4 *>(Qsrc), w32, donor, n_real, n_ghost);
 }
 void launch_max_dt(const double *w, const double *hmin, int64_t n, double gamma, unsigned long long *slot,
-                   cudaStream_t s, const int32_t *comp) {
-    if (n > 0) max_dt_kernel<<<blocks(n, 256), 256, 0, s>>>(w, hmin, n, gamma, slot, comp);
+                   cudaStream_t s, const int32_t *comp, const DtFinal &fin) {
+    if (n > 0 || fin.tstate) max_dt_kernel<<<blocks(n > 0 ? n : 1, kDtBlock), kDtBlock, 0, s>>>(w, hmin, n, gamma, slot, comp, fin);
 }
 
 namespace {
@@ -1665,11 +1754,6 @@ void launch_recip_check(const double *x, double *y, int64_t n, int which, cudaSt
 
 void launch_weno_coef32_check(const float4 *g, float *k, int64_t n, cudaStream_t s) {
     if (n > 0) weno_coef32_check_kernel<<<blocks(n, 256), 256, 0, s>>>(g, k, n);
-}
-
-void launch_dt_finalize(unsigned long long *slot, double *tstate, double cfl, double t_end,
-                        unsigned long long *nsteps, cudaStream_t s) {
-    dt_finalize_kernel<<<1, 1, 0, s>>>(slot, tstate, cfl, t_end, nsteps);
 }
 
 }  // namespace fdu

@@ -159,8 +159,8 @@ void launch_div_f32_tiles(const DivArgs &a, const TileTables &t, int mode, cudaS
 // *bad = min(*bad, first row of w[n][4] with rho <= 0 or a non-finite value)
 void launch_check_rows(const double *w, int64_t n, unsigned long long *bad, cudaStream_t s);
 void launch_permute_rows(const double *in, double *out, const int32_t *map, int64_t n, bool gather, cudaStream_t s);
-void launch_ghost_fill(double *w, const double *wsrc, void *F, const void *Fsrc, int fq, float4 *w32,
-                       const int32_t *donor, int64_t n_real, int64_t n_ghost, cudaStream_t s);
+void launch_ghost_fill(double *w, const double *wsrc, void *F, const void *Fsrc, int fq, double *Q, const double *Qsrc,
+                       float4 *w32, const int32_t *donor, int64_t n_real, int64_t n_ghost, cudaStream_t s);
 // FMA throughput (TFLOP/s) of `precision` 64 or 32 with sms*8 blocks of 256
 // threads; scratch holds sms*8*256 elements of that precision.
 double fma_probe_tflops(int precision, int sms, void *scratch, cudaStream_t s);
@@ -169,14 +169,19 @@ double fma_probe_tflops(int precision, int sms, void *scratch, cudaStream_t s);
 void launch_recip_check(const double *x, double *y, int64_t n, int which, cudaStream_t s);
 // k[24 i + j] = value j of the FP32 edge kernel's NU-WENO5 block formed from gaps g[i]
 void launch_weno_coef32_check(const float4 *g, float *k, int64_t n, cudaStream_t s);
-// Adaptive step: dt = min(cfl * bound, t_end - t) from the reduced bound in
-// *slot (bit pattern of a positive double); tstate = (t, dt, nonphysical);
-// the slot is reset to +inf for the next reduction; *nsteps counts steps
-// with dt > 0.
-void launch_dt_finalize(unsigned long long *slot, double *tstate, double cfl, double t_end,
-                        unsigned long long *nsteps, cudaStream_t s);
+// Adaptive step, finalised by the last block of the reduction: dt = min(cfl *
+// bound, t_end - t) from the reduced bound in *slot (bit pattern of a positive
+// double); tstate = (t, dt, nonphysical); the slot is reset to +inf for the next
+// reduction; *nsteps counts steps with dt > 0; *done counts the blocks (0
+// between launches).  tstate = nullptr: the reduction alone.
+struct DtFinal {
+    double *tstate;
+    double cfl, t_end;
+    unsigned long long *nsteps;
+    unsigned int *done;
+};
 void launch_max_dt(const double *w, const double *hmin, int64_t n, double gamma, unsigned long long *slot,
-                   cudaStream_t s, const int32_t *comp = nullptr);
+                   cudaStream_t s, const int32_t *comp = nullptr, const DtFinal &fin = DtFinal{});
 
 // One SSP-RK3 stage (mode 1..3) of a batch as one cooperative launch of
 // `blocks` x `threads` (edge fluxes, bounded grid barrier, divergence +
