@@ -15,6 +15,7 @@
 // fix band, |lambda|) take the same branch in the reverse pass.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "fdu_adjoint.cuh"
@@ -286,9 +287,7 @@ __device__ __forceinline__ dbl4 vertex_flux_vjp(const dbl4 &w, double gm1, const
 // (F_L + F_R)/2 - R |Lambda|_fixed L (w_R - w_L)/2 by Roe's property, so only
 // the left physical flux is differentiated.
 constexpr int kVjpBlock = 64;
-__global__ void __launch_bounds__(kVjpBlock) edge_flux_vjp_kernel(AdjEdgeArgs A) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= A.ne) return;
+__device__ __forceinline__ void edge_flux_vjp_body(const AdjEdgeArgs &A, const int64_t e, double (*wsm)[kVjpBlock]) {
     const double *__restrict__ w = A.w;
     const double *__restrict__ coef = A.coef;
     const double gm1 = A.gm1, hgm1 = 0.5 * A.gm1;
@@ -314,7 +313,6 @@ __global__ void __launch_bounds__(kVjpBlock) edge_flux_vjp_kernel(AdjEdgeArgs A)
     // each field's sub-stencil values and indicators and the combination's
     // products, kept in shared memory (thread-private column) for the
     // reverse sweep
-    __shared__ double wsm[4 * 22][kVjpBlock];
     const int t = threadIdx.x;
     auto keep = [&](int fi, const WenoField &W, const WenoKeep &K, const WenoHorner &H) {
         double *q = &wsm[fi * 22][t];
@@ -479,14 +477,28 @@ __global__ void __launch_bounds__(kVjpBlock) edge_flux_vjp_kernel(AdjEdgeArgs A)
     st4(G, 4 * ne + e, G4);
     st4(G, 5 * ne + e, G5);
 }
+__global__ void __launch_bounds__(kVjpBlock) edge_flux_vjp_kernel(const __grid_constant__ AdjEdgeArgs A) {
+    __shared__ double wsm[4 * 22][kVjpBlock];
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < A.ne) edge_flux_vjp_body(A, e, wsm);
+}
+// The edges the double-word kernel listed.
+__global__ void __launch_bounds__(kVjpBlock) edge_flux_vjp_list_kernel(const __grid_constant__ AdjEdgeArgs A) {
+    __shared__ double wsm[4 * 22][kVjpBlock];
+    const int n = *A.nlist;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        edge_flux_vjp_body(A, A.list[i], wsm);
+}
 
 // lam_r[k] = -sum_v we_vk lam_v (the table holds -we).  Thread i serves edge
 // perm[i]; its list is lane i % 32 of SELL-32 slice i / 32 (entry j at
 // off[slice] + 32 j + lane, padding with weight 0).
 __global__ void adj_edge_lambda_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ vid,
                                        const double *__restrict__ wt, const int32_t *__restrict__ perm,
-                                       const double *__restrict__ lam, double *__restrict__ lam_r, int64_t ne) {
+                                       const double *__restrict__ lam, double *__restrict__ lam_r, int64_t ne,
+                                       int *nlist) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (nlist && i == 0) *nlist = 0;
     if (i >= ne) return;
     const int64_t k = __ldg(perm + i);
     const int64_t sl = i / kSell;
@@ -582,9 +594,11 @@ void launch_ghost_fold(double *x, const int32_t *donor, const int64_t *off, cons
 void launch_residual_vjp(const AdjEdgeArgs &ea, const AdjTables &t, const AdjVertexArgs &va, cudaStream_t s) {
     if (ea.ne > 0) {
         adj_edge_lambda_kernel<<<nblk(ea.ne, 256), 256, 0, s>>>(t.eoff, t.evid, t.ewt, t.eperm, va.lam, ea.lam_r_mut,
-                                                               ea.ne);
-        if (ea.prec == 48) launch_edge_flux_vjp_dw(ea, s);
+                                                               ea.ne, ea.nlist);
+        if (ea.prec == 48 || ea.guard) launch_edge_flux_vjp_dw(ea, s);
         else edge_flux_vjp_kernel<<<nblk(ea.ne, kVjpBlock), kVjpBlock, 0, s>>>(ea);
+        if (ea.guard)  // at most four blocks on each of the 152 SMs
+            edge_flux_vjp_list_kernel<<<(unsigned)std::min<int64_t>(608, nblk(ea.ne, kVjpBlock)), kVjpBlock, 0, s>>>(ea);
     }
     if (va.nv > 0) adj_vertex_kernel<<<nblk(va.nv, 256), 256, 0, s>>>(va);
 }

@@ -16,8 +16,11 @@ struct AdjEdgeArgs {
     double *G;            // [6][ne][4] cotangents of the stencil states, per slot, then one zero record
     int64_t ne;
     double gm1, eps;
-    // precision 48 (double-word edge VJP, fdu_adjoint_dw.cu)
+    // double-word edge VJP (fdu_adjoint_dw.cu)
     int prec;              // 64 or 48
+    bool guard;            // precision 64 takes the edges it can in double words and lists the others
+    int32_t *list;         // [ne] listed edges
+    int *nlist;            // their count (reset by the transpose gather that runs before)
     const float4 *coefdw;  // [kDwPairs][ne] paired double-word coefficient block
     float dw_gm1[2], dw_tenth[2], dw_eps[2];
     int dw_eps_e;          // WENO epsilon = dw_eps * 2^dw_eps_e

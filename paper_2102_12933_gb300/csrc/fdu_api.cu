@@ -116,6 +116,8 @@ struct fdu_mesh {
     int32_t *adj_evid = nullptr, *adj_vvid = nullptr;
     int32_t *adj_eperm = nullptr, *adj_vperm = nullptr;  // thread -> edge / vertex of the transpose kernels
     double *adj_ewt = nullptr, *adj_wf = nullptr, *adj_wg = nullptr;
+    int32_t *adj_list = nullptr;      // edges the precision-64 double-word VJP left to FP64
+    int *adj_nlist = nullptr;
     double *adj_lam_r = nullptr, *adj_G = nullptr;
     double *adj_S1 = nullptr, *adj_buf[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     // transpose of the transmissive ghost fill: donors with their ghosts (CSR, internal ids)
@@ -818,6 +820,8 @@ fdu_status adjoint_setup(fdu_mesh *m) {
     // (the edge-flux VJP writes only the first 6 ne)
     if ((st = m->alloc(m->adj_G, 6 * 4 * ne + 4))) return st;
     CK(cudaMemset(m->adj_G, 0, (6 * 4 * ne + 4) * sizeof(double)));
+    if ((st = m->alloc(m->adj_list, ne))) return st;
+    if ((st = m->alloc(m->adj_nlist, 1))) return st;
     if ((st = m->alloc(m->adj_S1, 4 * nv))) return st;
     for (int i = 0; i < 5; ++i)
         if ((st = m->alloc(m->adj_buf[i], 4 * nv))) return st;
@@ -869,7 +873,14 @@ void enqueue_residual_vjp(fdu_mesh *m, const double *w, const double *lam, doubl
     ea.gm1 = m->opts.gamma - 1.0;
     ea.eps = m->opts.weno_eps;
     ea.prec = m->adj_prec;
-    if (m->adj_prec == 48) {
+    // precision 64: double words where the WENO epsilon can reach the guard's
+    // 2^-76 E^2 for energies of their window (2^-24 and up), FP64 otherwise
+    ea.guard = m->adj_prec == 64 && m->dw64 && m->opts.weno_eps >= 0x1p-124;
+    if (ea.guard) {
+        ea.list = m->adj_list;
+        ea.nlist = m->adj_nlist;
+    }
+    if (m->adj_prec == 48 || ea.guard) {
         const EdgeArgs e48 = edge_args(m, 48, w);
         ea.coefdw = e48.coefdw;
         for (int i = 0; i < 2; ++i) {
