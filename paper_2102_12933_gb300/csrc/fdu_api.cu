@@ -91,7 +91,7 @@ struct fdu_mesh {
                                              // [4] stage updates scaled by the positivity safeguard,
                                              // [5] first non-physical row of a state being set
     // adaptive stepping: (t, dt, nonphysical flag), then the step counter and
-    // the wide flags in the fourth to sixth words, all reset by one memset
+    // the wide flags in the fourth to sixth words, all reset with the state
     double *tstate = nullptr;
     unsigned long long *nsteps = nullptr;    // adaptive steps taken (in tstate's fourth word)
     int *wide = nullptr;                     // [kWideSlots] (in tstate's fifth and sixth words)
@@ -1178,7 +1178,7 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
     if (!w) return set_err(FDU_ERR_ARG, "null state");
     cudaStream_t s = m->stream(stream);
     if (on_device) {
-        launch_permute_rows(w, m->wn, m->new2old, m->nv, true, s);
+        launch_permute_rows(w, m->wn, m->new2old, m->nv, true, s, m->tstate, kTState);
         CK_LAUNCH();
     } else {
         // one copy of the caller's rows (a DMA when they are pinned), checked
@@ -1194,7 +1194,7 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
         CK(cudaStreamSynchronize(s));
         if (bad != none)
             return set_err(FDU_ERR_NONPHYSICAL, "state row " + std::to_string(bad) + " has rho <= 0 or a non-finite value");
-        launch_permute_rows(m->scratch, m->wn, m->new2old, m->nv, true, s);
+        launch_permute_rows(m->scratch, m->wn, m->new2old, m->nv, true, s, m->tstate, kTState);
         CK_LAUNCH();
     }
     if (m->n_ghost > 0) {
@@ -1203,7 +1203,6 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
         CK_LAUNCH();
     }
     m->f64_valid = m->f32_valid = false;
-    CK(cudaMemsetAsync(m->tstate, 0, kTState * sizeof(double), s));
     return FDU_OK;
 }
 
