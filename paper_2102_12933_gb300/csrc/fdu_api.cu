@@ -130,10 +130,14 @@ struct fdu_mesh {
     std::vector<cudaEvent_t> prof_ev[6];
     size_t prof_used[6] = {0, 0, 0, 0, 0, 0};
 
-    // Device memory of the mesh, freed with it.  Requests up to kSmall share
-    // chunks: a cudaMalloc takes tens of microseconds, and a small mesh makes
-    // about fifty requests.
-    static constexpr size_t kSmall = 256 << 10, kChunk = 4 << 20, kAlign = 256;
+    // Device memory of the mesh, freed with it.  Small requests share chunks: a
+    // cudaMalloc takes tens of microseconds, and a mesh makes about sixty
+    // requests.  A chunk is as large as half of what the mesh holds already
+    // (within kChunkMin and kChunkMax), and requests up to a quarter of that
+    // share it, so that what stays unused is a fraction of the mesh's own size.
+    // Creation of 3600 and 10,000 vertices: 9.3 and 21.1 ms with chunks of 4 MB
+    // for requests up to 256 KB, 9.0 and 20.5 ms so.
+    static constexpr size_t kChunkMin = 4 << 20, kChunkMax = 64 << 20, kAlign = 256;
     char *chunk = nullptr;
     size_t chunk_left = 0;
     template <class T>
@@ -141,22 +145,24 @@ struct fdu_mesh {
         p = nullptr;
         if (count == 0) count = 1;
         const size_t bytes = (count * sizeof(T) + kAlign - 1) / kAlign * kAlign;
-        void *q = nullptr;
-        if (bytes > kSmall || bytes > chunk_left) {
-            const size_t take = bytes > kSmall ? bytes : kChunk;
+        const size_t next = std::clamp((size_t)device_bytes / 2 / kAlign * kAlign, kChunkMin, kChunkMax);
+        if (bytes > chunk_left || bytes > next / 4) {
+            void *q = nullptr;
+            const size_t take = bytes > next / 4 ? bytes : next;
             cudaError_t e = cudaMalloc(&q, take);
             if (e != cudaSuccess) return set_err(FDU_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
             allocs.push_back(q);
-            if (bytes <= kSmall) {
-                chunk = static_cast<char *>(q);
-                chunk_left = take;
+            if (bytes > next / 4) {
+                device_bytes += (int64_t)(count * sizeof(T));
+                p = static_cast<T *>(q);
+                return FDU_OK;
             }
+            chunk = static_cast<char *>(q);
+            chunk_left = take;
         }
-        if (bytes <= kSmall) {
-            q = chunk;
-            chunk += bytes;
-            chunk_left -= bytes;
-        }
+        void *q = chunk;
+        chunk += bytes;
+        chunk_left -= bytes;
         device_bytes += (int64_t)(count * sizeof(T));
         p = static_cast<T *>(q);
         return FDU_OK;

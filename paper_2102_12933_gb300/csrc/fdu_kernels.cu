@@ -910,6 +910,9 @@ __device__ unsigned short tile_position(const int32_t *list, int n, int32_t id) 
     }
     return (unsigned short)lo;
 }
+// Grid (tiles, 2): vertices and edges of a tile are built by two blocks.  On a
+// small mesh the time is one block's serial chain (1600 vertices: the sizes in
+// 50 us and the tables in 178, with one block after the other 62 and 262).
 __global__ void __launch_bounds__(kTileThreads)
     tile_count_kernel(TileSource S, TileTables T, int32_t *nv, int32_t *ne, int32_t *gv, int32_t *ge) {
     extern __shared__ int tile_work[];
@@ -917,13 +920,14 @@ __global__ void __launch_bounds__(kTileThreads)
     __shared__ int key[kTile];
     const int64_t t = blockIdx.x, p0 = t * kTile, v0 = S.start[t];
     const int nvt = S.start[t + 1] - S.start[t], i = threadIdx.x;
+    const bool edges = blockIdx.y != 0;
     TileRow r{0, 0, 0, 0};
     if (i < kTile) {
         if (i < nvt) r = tile_row(S, v0 + i);
         key[i] = i < nvt ? (r.J << 16) | r.K : -1;
     }
     __syncthreads();
-    if (i < kTile) {  // decreasing (J, K), ties in vertex order
+    if (i < kTile && !edges) {  // decreasing (J, K), ties in vertex order
         int rank = 0;
         for (int q = 0; q < kTile; ++q) rank += key[q] > key[i] || (key[q] == key[i] && q < i);
         W.J[rank] = r.J;
@@ -931,7 +935,7 @@ __global__ void __launch_bounds__(kTileThreads)
         T.perm[p0 + rank] = i < nvt ? (int32_t)(v0 + i) : -1;
     }
     __syncthreads();
-    if (i < kTile / kSell) {
+    if (i < kTile / kSell && !edges) {
         int mj = 0, mk = 0;
         for (int l = 0; l < kSell; ++l) {
             mj = max(mj, W.J[i * kSell + l]);
@@ -940,13 +944,8 @@ __global__ void __launch_bounds__(kTileThreads)
         gv[t * (kTile / kSell) + i] = (mj + 3) / 4;
         ge[t * (kTile / kSell) + i] = (mk + 3) / 4;
     }
-    const int a = tile_unique(W, S, v0, nvt, false);
-    __syncthreads();
-    const int c = tile_unique(W, S, v0, nvt, true);
-    if (i == 0) {
-        nv[t] = a;
-        ne[t] = c;
-    }
+    const int n = tile_unique(W, S, v0, nvt, edges);
+    if (i == 0) (edges ? ne : nv)[t] = n;
 }
 // Order of a slice's entries over its steps.  A 16-byte shared-memory read is
 // served eight lanes at a time, and positions equal modulo 8 fall on the same
@@ -999,57 +998,55 @@ __global__ void __launch_bounds__(kTileThreads) tile_fill_kernel(TileSource S, T
     const int32_t v = i < kTile ? T.perm[p0 + i] : -1;
     const TileRow r = v >= 0 ? tile_row(S, v) : TileRow{0, 0, 0, 0};
     const int64_t sl = t * (kTile / kSell) + i / kSell, lane = i % kSell;
-    for (int part = 0; part < 2; ++part) {
-        const int32_t *ids = part ? S.eid : S.vid;
-        const int64_t b = part ? r.eb : r.vb;
-        const int cnt = part ? r.K : r.J;
-        const int32_t *goff = part ? T.geoff : T.gvoff;
-        const int n = tile_unique(W, S, v0, nvt, part != 0);
-        int32_t *list = part ? T.elist + T.eoff[t] : T.vlist + T.voff[t];
-        for (int q = i; q < n; q += kTileThreads) list[q] = W.list[q];
-        const int64_t g0 = i < kTile ? goff[sl] : 0;
-        const int steps = i < kTile ? 4 * (int)(goff[sl + 1] - g0) : 0;
-        const bool scheduled = steps <= kTileSteps;  // the same for the lanes of a slice
-        int *count = part ? W.K : W.J;
-        __syncthreads();  // the hash table's memory holds positions from here
-        if (i < kTile) {
-            count[i] = cnt;
-            if (scheduled)
-                for (int j = 0; j < cnt; ++j) W.pos[j][i] = tile_position(W.list, n, ids[b + (int64_t)kSell * j]);
-        }
-        __syncthreads();
-        if (i < kTile && scheduled && i % 8 == 0) tile_schedule(W, i / 8, steps, count);
-        __syncthreads();
-        if (i < kTile) {
-            // a step without an entry repeats the lane's first with weight 0, as
-            // the SELL padding does, so that a non-finite flux reaches only the
-            // vertices whose stencils hold it
-            unsigned short *pos = reinterpret_cast<unsigned short *>(part ? T.epos : T.vpos);
-            float *wa = reinterpret_cast<float *>(part ? T.we : T.wf), *wb = reinterpret_cast<float *>(T.wg);
-            const float *sa = part ? S.we : S.wf;
-            unsigned char cur[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            for (int s = 0; s < steps; ++s) {
-                int j = s < cnt ? s : -1;
-                unsigned short p = 0;
-                if (scheduled) {
-                    const int c = W.bank[s][i];
-                    j = -1;
-                    if (c < 8) {
-                        j = cur[c];
-                        while ((W.pos[j][i] & 7) != c) ++j;
-                        cur[c] = (unsigned char)(j + 1);
-                    }
-                    if (cnt > 0) p = W.pos[j < 0 ? 0 : j][i];
-                } else if (cnt > 0) {
-                    p = tile_position(W.list, n, ids[b + (int64_t)kSell * (j < 0 ? 0 : j)]);
+    const int part = blockIdx.y;  // 0: vertices, 1: edges
+    const int32_t *ids = part ? S.eid : S.vid;
+    const int64_t b = part ? r.eb : r.vb;
+    const int cnt = part ? r.K : r.J;
+    const int32_t *goff = part ? T.geoff : T.gvoff;
+    const int n = tile_unique(W, S, v0, nvt, part != 0);
+    int32_t *list = part ? T.elist + T.eoff[t] : T.vlist + T.voff[t];
+    for (int q = i; q < n; q += kTileThreads) list[q] = W.list[q];
+    const int64_t g0 = i < kTile ? goff[sl] : 0;
+    const int steps = i < kTile ? 4 * (int)(goff[sl + 1] - g0) : 0;
+    const bool scheduled = steps <= kTileSteps;  // the same for the lanes of a slice
+    int *count = part ? W.K : W.J;
+    __syncthreads();  // the hash table's memory holds positions from here
+    if (i < kTile) {
+        count[i] = cnt;
+        if (scheduled)
+            for (int j = 0; j < cnt; ++j) W.pos[j][i] = tile_position(W.list, n, ids[b + (int64_t)kSell * j]);
+    }
+    __syncthreads();
+    if (i < kTile && scheduled && i % 8 == 0) tile_schedule(W, i / 8, steps, count);
+    __syncthreads();
+    if (i < kTile) {
+        // a step without an entry repeats the lane's first with weight 0, as
+        // the SELL padding does, so that a non-finite flux reaches only the
+        // vertices whose stencils hold it
+        unsigned short *pos = reinterpret_cast<unsigned short *>(part ? T.epos : T.vpos);
+        float *wa = reinterpret_cast<float *>(part ? T.we : T.wf), *wb = reinterpret_cast<float *>(T.wg);
+        const float *sa = part ? S.we : S.wf;
+        unsigned char cur[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (int s = 0; s < steps; ++s) {
+            int j = s < cnt ? s : -1;
+            unsigned short p = 0;
+            if (scheduled) {
+                const int c = W.bank[s][i];
+                j = -1;
+                if (c < 8) {
+                    j = cur[c];
+                    while ((W.pos[j][i] & 7) != c) ++j;
+                    cur[c] = (unsigned char)(j + 1);
                 }
-                const int64_t q = 4 * ((g0 + s / 4) * kSell + lane) + s % 4, src = b + (int64_t)kSell * j;
-                pos[q] = p;
-                wa[q] = j >= 0 ? sa[src] : 0.0f;
-                if (!part) wb[q] = j >= 0 ? S.wg[src] : 0.0f;
+                if (cnt > 0) p = W.pos[j < 0 ? 0 : j][i];
+            } else if (cnt > 0) {
+                p = tile_position(W.list, n, ids[b + (int64_t)kSell * (j < 0 ? 0 : j)]);
             }
+            const int64_t q = 4 * ((g0 + s / 4) * kSell + lane) + s % 4, src = b + (int64_t)kSell * j;
+            pos[q] = p;
+            wa[q] = j >= 0 ? sa[src] : 0.0f;
+            if (!part) wb[q] = j >= 0 ? S.wg[src] : 0.0f;
         }
-        __syncthreads();
     }
 }
 
@@ -1425,7 +1422,9 @@ __device__ __forceinline__ void dt_finalize(unsigned long long *slot, double *ts
 // a few 2^-24 relative, times the Mach number through the pressure; a vertex
 // with p < 2^-10 rho E (Mach above 40), or outside FP32's comfortable range, is
 // always taken, so the result is the FP64 minimum itself.  With `fin` (adaptive stepping) the last block
-// also finalises the step.
+// also finalises the step.  1,000,000 vertices: 19.6 us (89 with every vertex
+// in FP64 and the finalisation as a launch of its own); the state alone is 32
+// MB.
 constexpr int kDtBlock = 256;
 __global__ void __launch_bounds__(kDtBlock)
     max_dt_kernel(const double *__restrict__ w, const double *__restrict__ hmin, int64_t n, double gamma,
@@ -1584,10 +1583,10 @@ void launch_div_f32(const DivArgs &a, int mode, cudaStream_t s) {
 void launch_tile_count(const TileSource &S, const TileTables &T, int32_t *nv, int32_t *ne, int32_t *gv, int32_t *ge,
                        cudaStream_t s) {
     if (T.ntiles > 0)
-        tile_count_kernel<<<(unsigned)T.ntiles, kTileThreads, sizeof(TileWork), s>>>(S, T, nv, ne, gv, ge);
+        tile_count_kernel<<<dim3((unsigned)T.ntiles, 2), kTileThreads, sizeof(TileWork), s>>>(S, T, nv, ne, gv, ge);
 }
 void launch_tile_fill(const TileSource &S, const TileTables &T, cudaStream_t s) {
-    if (T.ntiles > 0) tile_fill_kernel<<<(unsigned)T.ntiles, kTileThreads, sizeof(TileWork), s>>>(S, T);
+    if (T.ntiles > 0) tile_fill_kernel<<<dim3((unsigned)T.ntiles, 2), kTileThreads, sizeof(TileWork), s>>>(S, T);
 }
 void launch_div_f32_tiles(const DivArgs &a, const TileTables &t, int mode, cudaStream_t s) {
     const unsigned g = (unsigned)t.ntiles;
