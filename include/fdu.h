@@ -293,11 +293,14 @@ fdu_status fdu_batch_barrier_selftest(fdu_mesh *batch, int *status);
  * respect to its fixed value.  fdu_rk_step_vjp and fdu_adjoint_rk return
  * FDU_ERR_ARG when the stage positivity safeguard is on (positivity_alpha
  * > 0): the safeguard is not differentiated. */
-/* Precision of the adjoint calls below: 64 (FP64, the default) or 48.  With
- * 48 the edge-flux VJP runs in double-word FP32 (the same derivative to about
+/* Precision of the adjoint calls below: 64 (the default) or 48.  With 48 the
+ * edge-flux VJP runs in double-word FP32 (the same derivative to about
  * 1e-13, on the FP32 pipes) and the steps that fdu_rk_step_vjp and
  * fdu_adjoint_rk take or recompute are precision-48 steps (the trajectory of
- * fdu_rk_step(..., 48)).  The first use of 48 builds its tables. */
+ * fdu_rk_step(..., 48)).  With 64 the steps are precision-64 steps and the
+ * double-word VJP serves the edges where it holds FP64's accuracy, which
+ * takes weno_eps >= 2^-124; every other edge, and every edge below that
+ * epsilon, is differentiated in FP64. */
 fdu_status fdu_set_adjoint_precision(fdu_mesh *mesh, int precision);
 /* grad = (dL/dw)^T lam at the current state. */
 fdu_status fdu_residual_vjp(fdu_mesh *mesh, const double *lam, double *grad, int on_device, void *stream);
