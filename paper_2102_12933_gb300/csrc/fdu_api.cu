@@ -95,6 +95,7 @@ struct fdu_mesh {
     double *tstate = nullptr;
     unsigned long long *nsteps = nullptr;    // adaptive steps taken (in tstate's fourth word)
     int *wide = nullptr;                     // [kWideSlots] (in tstate's fifth and sixth words)
+    bool wide_clean = false;                 // no launch has set or could have set a wide flag since they were zeroed
     bool f64_valid = false, f32_valid = false;              // F64[0] / (w32, F32[0]) describe wn
     cudaStream_t own_stream = nullptr;
     std::map<std::pair<int, double>, cudaGraphExec_t> graphs;
@@ -623,9 +624,13 @@ void timed(fdu_mesh *m, int kind, bool allowed, cudaStream_t s, F &&launch) {
     if (p) cudaEventRecord(p[1], s);
 }
 
-// Make F64[0] (or w32 and F32[0]) describe the current state wn.
+// Make F64[0] (or w32 and F32[0]) describe the current state wn.  The wide flags
+// are zeroed first where calls since fdu_set_state (which zeroes them in its own
+// launch) can have left some, so that they depend on the state alone.
 void ensure_fluxes(fdu_mesh *m, int prec, cudaStream_t s) {
     if (fp64_state(prec) && !m->f64_valid) {
+        if (!m->wide_clean) cudaMemsetAsync(m->wide, 0, kWideSlots * sizeof(int), s);
+        m->wide_clean = false;
         launch_vertex_flux_f64(m->wn, m->F64[0], m->nv, m->opts.gamma, s, m->Q64[0], m->wide, m->n_real);
         m->f64_valid = true;
     }
@@ -1209,6 +1214,7 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
         CK_LAUNCH();
     }
     m->f64_valid = m->f32_valid = false;
+    m->wide_clean = true;
     return FDU_OK;
 }
 

@@ -126,9 +126,13 @@ __device__ __forceinline__ dw2 ld_dw2(const Stage &T, int j) {
     return dw2{pk(q.x, q.y), pk(q.z, q.w)};
 }
 
-// The slot that the next stage writes (nothing reads it any more).
+// The slots that the first two stages write, cleared in the first stage, and the
+// slot of the step's result, cleared in the third stage just before that stage
+// writes it: a caller may stop after the second stage and keep the start state.
 __device__ __forceinline__ void clear_wide(const EdgeArgs &A, int64_t e) {
-    if (A.wide && e == 0) A.wide[A.wide_in == 0 ? 2 : A.wide_in - 1] = 0;
+    if (!A.wide || e != 0) return;
+    if (A.wide_in == 0) A.wide[1] = A.wide[2] = 0;
+    if (A.wide_in == 2) A.wide[0] = 0;
 }
 
 // Writes the increment of edge e and returns true.  With GUARD (precision 64)

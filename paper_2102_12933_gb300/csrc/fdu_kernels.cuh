@@ -16,9 +16,10 @@ constexpr int kDivBlock = 128;   // threads per block, divergence kernels
 // so that squares and products of the edge flux stay far from 2^+-126.  wide[i]
 // is non-zero when the state of flux buffer i (0..2) failed, wide[3] when a
 // ghost of the state that was set did (Dirichlet ghosts keep it).  A stage
-// that finds wide[in] or wide[3] set runs in FP64 throughout; the edge kernel
-// of each stage clears the slot that the stage after it writes (the buffers
-// rotate, and nothing reads that slot in between).
+// that finds wide[in] or wide[3] set runs in FP64 throughout.  The edge kernels
+// clear the slots (clear_wide): the first stage's those of the two intermediate
+// states, the third stage's that of the result, so that the flag of a state
+// whose step is only partly taken (the adjoint's recomputation) stands.
 constexpr int kWideGhost = 3;
 constexpr int kWideSlots = 4;
 constexpr int kWideExp = 24;
