@@ -287,7 +287,8 @@ __device__ __forceinline__ double scaled_down(double x, int k) {
 }
 
 // GUARD (precision 64): returns false, writing nothing, for an edge that FP64
-// takes: a state outside the forward kernel's window, an average whose c^2 is a
+// takes: a state outside the forward kernel's density and energy window,
+// differences that are not finite in FP32 (a NaN or huge momentum), an average whose c^2 is a
 // small difference (edge_flux_dw_body), a cotangent that is not finite, or a
 // WENO epsilon so far below the state's squares that the derivative of the
 // weights rests on the rounding of the differences (eps < 2^-76 E^2: noise of
@@ -304,10 +305,11 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     const dw2 nn = ldk(kp, ne, kDwPairs - 1);
     const dw nx = first(nn), ny = second(nn);
 
-    // the cotangent scaled by the power of two that brings its largest component to [1, 2)
+    // the cotangent scaled by the power of two that brings its largest component to
+    // [1, 2); as it is where one is not finite, which the split passes on
     d4v lam = ldd4(A.lam_r, e);
     const int big = max(max(dexp(lam.x), dexp(lam.y)), max(dexp(lam.z), dexp(lam.w)));
-    const int kl = big - 1023;
+    const int kl = big == 2047 ? 0 : big - 1023;
     if (GUARD && (big == 2047 || (big == 0 && (lam.x != 0.0 || lam.y != 0.0 || lam.z != 0.0 || lam.w != 0.0)))) return false;
     lam = d4v{scaled_down(lam.x, kl), scaled_down(lam.y, kl), scaled_down(lam.z, kl), scaled_down(lam.w, kl)};
 
@@ -353,8 +355,11 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     const Roe2 C = roe2(W1, P1, gm1);
     if (GUARD && !(C.R.H.h - C.R.hq2.h >= 0.25f * C.R.H.h)) return false;
     {
+        f2 finite = pk(0.0f, 0.0f);  // 0 while every field is
         auto put = [&](const vec4<f2> &d, int slot) {
             const vec4<f2> c = project_n(C.R, d);
+            const f2 z = pk(0.0f, 0.0f);
+            if (GUARD) finite = ffma(c.x.h, z, ffma(c.n.h, z, ffma(c.t.h, z, ffma(c.w.h, z, finite))));
             st_dw2(S, slot, norm(c.x));
             st_dw2(S, slot + 1, norm(c.n));
             st_dw2(S, slot + 2, norm(c.t));
@@ -362,6 +367,7 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
         };
         put(dpair(s[1], s[4]), kSlotBF);
         put(dpair(s[0], s[5]), kSlotAE);
+        if (GUARD && !(lane0(finite) == 0.0f && lane1(finite) == 0.0f)) return false;
         const vec4<float> c = project_n(C.R, dmid());
         st_dw2(S, kSlotC, norm(pair(c.x, c.n)));
         st_dw2(S, kSlotC + 1, norm(pair(c.t, c.w)));
@@ -465,7 +471,11 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     double *G = A.G;  // [6][ne][4]
     auto put = [&](int slot, dw x, dw n, dw t, dw v) {  // back to x-y components and to FP64, unscaled
         const dw2 m = norm(lfma(pair(lneg(ny), nx), both(t), lmul(pair(nx, ny), both(n))));
-        auto to = [&](float h, float l) { return f2d_scaled(h, kl) + f2d_scaled(l, kl); };
+        auto to = [&](float h, float l) {
+            const double v = f2d_scaled(h, kl) + f2d_scaled(l, kl);
+            const bool finite = (__float_as_uint(h) & 0x7f800000u) != 0x7f800000u;
+            return finite ? v : __hiloint2double(0x7ff80000, 0);
+        };
         double2 *q = reinterpret_cast<double2 *>(G + 4 * ((int64_t)slot * ne + e));
         q[0] = make_double2(to(x.h, x.l), to(lane0(m.h), lane0(m.l)));
         q[1] = make_double2(to(lane1(m.h), lane1(m.l)), to(v.h, v.l));

@@ -131,25 +131,27 @@ __device__ __forceinline__ dw dot2_result(const dot2 &A) { return two_sum(A.s, A
 // stay far above); the high word keeps the top 24 bits (truncated), the low
 // word the next 24 of the remaining 29 (relative error below 2^-47).  The
 // pair is not renormalised (|l| < ulp(h) instead of ulp(h)/2): the
-// operations that take it renormalise their results.
+// operations that take it renormalise their results.  Magnitudes of 2^128 and
+// above, infinities and NaN give an infinity or a NaN.
 __device__ __forceinline__ dw d2dw(double d) {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
     const int e = (int)((hi >> 20) & 0x7ffu);
     if (e <= 896) return dw_make(0.0f, 0.0f);
     const unsigned sgn = hi & 0x80000000u;
-    const float h = __uint_as_float(sgn | ((unsigned)(e - 896) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    const float h = __uint_as_float(sgn | ((unsigned)min(e - 896, 255) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
     const unsigned m = lo & 0x1fffffffu;  // value m 2^(e - 1075)
     const unsigned lb = __float_as_uint(__uint2float_rn(m));
     const int le = (int)((lb >> 23) & 0xffu) + (e - 1075);
     const float l = (m != 0u && le > 0) ? __uint_as_float(sgn | ((unsigned)le << 23) | (lb & 0x7fffffu)) : 0.0f;
     return dw_make(h, l);  // |l| < ulp(h): the truncated split, not renormalised
 }
-// float -> double, exact for normal floats (zero and subnormals -> 0)
+// float -> double, exact for normal floats (zero and subnormals -> 0; infinities
+// and NaN stay what they are)
 __device__ __forceinline__ double f2d(float x) {
     const unsigned b = __float_as_uint(x);
-    const unsigned e = (b >> 23) & 0xffu;
+    const unsigned e = (b >> 23) & 0xffu, d = e == 255u ? 2047u : e + 896u;
     if (e == 0u) return 0.0;
-    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
+    return __hiloint2double((int)((b & 0x80000000u) | (d << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
 }
 
 

@@ -149,10 +149,12 @@ __device__ __forceinline__ bool stage_is_wide(const int *wide, int in) {
 }
 // A state outside the double words' window: density or energy not in
 // [2^-kWideExp, 2^kWideExp), by the exponent field (NaN, zero, negative and
-// infinite values fail).
-__device__ __forceinline__ bool outside_window(const dbl4 &w) {
+// infinite values fail), or a pressure p that is not positive (the momentum then
+// has |m|^2 < 2 rho E, so it is in range too; a NaN or infinite one gives a NaN or
+// -infinite pressure).
+__device__ __forceinline__ bool outside_window(const dbl4 &w, double p) {
     const unsigned lo = (unsigned)(1023 - kWideExp) << 20, n = (unsigned)(2 * kWideExp) << 20;
-    return (unsigned)__double2hiint(w.x) - lo >= n || (unsigned)__double2hiint(w.w) - lo >= n;
+    return (unsigned)__double2hiint(w.x) - lo >= n || (unsigned)__double2hiint(w.w) - lo >= n || !pos64(p);
 }
 
 // ------------------------------------------------------------------ vertex fluxes
@@ -180,7 +182,7 @@ __global__ void vertex_flux_f64_kernel(const double *__restrict__ w, double *__r
     st4(F, 2 * v, f);
     st4(F, 2 * v + 1, g);
     if (Q) st4(Q, v, roe_record64(s, P));
-    if (wide && outside_window(s)) wide[v < n_real ? 0 : kWideGhost] = 1;
+    if (wide && outside_window(s, P.p)) wide[v < n_real ? 0 : kWideGhost] = 1;
 }
 
 // Forward-Euler part of an SSP-RK3 stage, fe = ws + theta dt L.  Without
@@ -363,7 +365,7 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i, 
     st4(Fo, 2 * v, f);
     st4(Fo, 2 * v + 1, g);
     if (A.Qout) st4(A.Qout, v, roe_record64(o, P));
-    if (A.wide && outside_window(o)) A.wide[A.wide_out] = 1;
+    if (A.wide && outside_window(o, P.p)) A.wide[A.wide_out] = 1;
 }
 // The FP64 form out of line, for the kernels that seldom take it.
 template <int MODE>

@@ -12,8 +12,9 @@ constexpr int kDivBlock = 128;   // threads per block, divergence kernels
 
 // Precision 64 takes an edge's increments in double words where FP32's exponent
 // range holds them.  The kernels that write a state's fluxes (vertex_flux, the
-// stage epilogues) check every vertex: density and energy within 2^+-kWideExp,
-// so that squares and products of the edge flux stay far from 2^+-126.  wide[i]
+// stage epilogues) check every vertex: density and energy within 2^+-kWideExp
+// and a positive pressure, which bounds the momentum, so that squares and
+// products of the edge flux stay far from 2^+-126 and no NaN or infinity is there.  wide[i]
 // is non-zero when the state of flux buffer i (0..2) failed, wide[3] when a
 // ghost of the state that was set did (Dirichlet ghosts keep it).  A stage
 // that finds wide[in] or wide[3] set runs in FP64 throughout.  The edge kernels
