@@ -367,9 +367,16 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i, 
     if (A.Qout) st4(A.Qout, v, roe_record64(o, P));
     if (A.wide && outside_window(o, P.p)) A.wide[A.wide_out] = 1;
 }
-// The FP64 form out of line, for the kernels that seldom take it.
-template <int MODE>
-__device__ __noinline__ void div_f64_cold(const DivArgs *A, const int64_t i) { div_f64_body<MODE, false>(*A, i); }
+// The FP64 form out of line, for the kernels that seldom take it.  It shares a
+// vertex between the same lanes: RK3 step outside the window with one of them at
+// work / all / in the FP64 kernels alone, one lane to a vertex: 10,000 vertices
+// 238 / 163 / 186 us, 22,500 347 / 294 / 294, 55,225 719 / 610 / 578 (the stage
+// update of one lane in two takes a warp's FP64 time; a vertex to each thread of
+// half the block gives 606 there, and 240 for 222 us at 14,400).
+template <int MODE, int LPV>
+__device__ __noinline__ void div_f64_cold(const DivArgs *A, const int64_t i, const int q, const bool on) {
+    div_f64_body<MODE, false, LPV>(*A, i, q, on);
+}
 // The divergence of one vertex by KIND (kDivPlain, kDivDw, kDivGuard).
 template <int MODE, int KIND, int LPV = 1>
 __device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, const bool wide, const int q = 0,
@@ -377,7 +384,7 @@ __device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, c
     if (KIND == kDivPlain) {
         div_f64_body<MODE, false, LPV>(A, i, q, on);
     } else if (KIND == kDivGuard && wide) {
-        if (q == 0 && on) div_f64_cold<MODE>(&A, i);
+        div_f64_cold<MODE, LPV>(&A, i, q, on);
     } else {
         div_f64_body<MODE, true, LPV>(A, i, q, on);
     }

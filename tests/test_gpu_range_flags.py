@@ -37,3 +37,27 @@ def test_step_vjp_leaves_the_flags_of_its_state(s, adjoint):
     M.rk_step_vjp(dt, lam)
     M.rk_step(dt, 64)
     assert np.array_equal(M.get_state(), stepped)
+
+
+@pytest.mark.parametrize("n", [16, 110, 111, 240])
+def test_wide_state_over_the_lanes_of_a_vertex(n):
+    """FP64 throughout with four (to 12,288 vertices), two (to 57,344) and one
+    lane to a vertex: fdu_residual_noalloc to 1e-13 (the same sums, without
+    the vertices' Roe records), and a step in density units of 2^40 to the parity bound
+    1e-11 of the increment."""
+    s = 2.0 ** 40
+    m, w = inputs.vortex_case(n, seed=n)
+    M = fdu.Mesh(m.xy, m.tri, m.Lx, m.Ly, weno_eps=1e-300)
+    t = torch.tensor(w * s, device="cuda")
+    want, got = torch.empty_like(t), torch.empty_like(t)
+    M.residual_noalloc(t, want)
+    M.set_state(t)
+    M.residual(64, out=got)
+    assert float(torch.linalg.norm(got - want) / torch.linalg.norm(want)) <= 1e-13
+    dt = M.max_dt(0.4)
+    M.rk_step(dt, 64)
+    wide = M.get_state() / s
+    M.set_state(w)
+    M.rk_step(dt, 64)
+    one = M.get_state()
+    assert np.linalg.norm(wide - one) <= 1e-11 * np.linalg.norm(one - w)
