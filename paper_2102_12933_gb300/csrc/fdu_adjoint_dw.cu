@@ -286,13 +286,18 @@ __device__ __forceinline__ double scaled_down(double x, int k) {
     return __hiloint2double((__double2hiint(x) & (int)0x800fffff) | (e << 20), __double2loint(x));
 }
 
-// GUARD (precision 64): returns false, writing nothing, for an edge that FP64
-// takes: a state outside the forward kernel's density and energy window,
+// GUARD (precision 64): returns false for an edge that FP64 takes and writes: a state outside the forward kernel's density and energy window,
 // differences that are not finite in FP32 (a NaN or huge momentum), an average whose c^2 is a
 // small difference (edge_flux_dw_body), a cotangent that is not finite, or a
 // WENO epsilon so far below the state's squares that the derivative of the
 // weights rests on the rounding of the differences (eps < 2^-76 E^2: noise of
-// 2^-53 of the state, squared, would pass for an indicator).
+// 2^-53 of the state, squared, would pass for an indicator), or end states more
+// than a factor of two apart in density or energy.  VJP against central
+// differences in extended precision, FP64 / double words without the last line /
+// with it, steps of 4, 16, 64 in density and pressure: 7.7e-14 / 1.4e-13 / 3.1e-14,
+// 4.7e-14 / 2.6e-13 / 5.5e-14, 6.8e-14 / 3.9e-13 / 6.5e-14.  A line at 1.5 lists
+// edges of smooth flow on coarse meshes (beta 5 vortex on 24^2 and 40^2: 71 and 75
+// to 113 us) and gains nothing.
 template <bool GUARD>
 __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int64_t e, const Stage &S) {
     const double *__restrict__ w = A.w;
@@ -316,11 +321,14 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     // ---------------- forward
     const d4v L1d = ldd4(w, s[2]), R1d = ldd4(w, s[3]);
     if (GUARD) {
-        auto out = [](const d4v &q) {
-            const unsigned lo = (unsigned)(1023 - kWideExp) << 20, n = (unsigned)(2 * kWideExp) << 20;
-            return (unsigned)__double2hiint(q.x) - lo >= n || (unsigned)__double2hiint(q.w) - lo >= n;
-        };
+        // the high words of positive doubles order them, and 2^20 between two of them
+        // is a factor of two
+        const unsigned lo = (unsigned)(1023 - kWideExp) << 20, n = (unsigned)(2 * kWideExp) << 20;
+        auto hi = [](double x) { return (unsigned)__double2hiint(x); };
+        auto out = [&](const d4v &q) { return hi(q.x) - lo >= n || hi(q.w) - lo >= n; };
+        auto jump = [&](double a, double b) { return hi(a) - hi(b) + (1u << 20) > 1u << 21; };
         bool bad = out(L1d) || out(R1d) || dexp(A.eps) < 2 * dexp(L1d.w) - 1023 - 76;
+        bad = bad || jump(L1d.x, R1d.x) || jump(L1d.w, R1d.w);
         bad = bad || out(ldd4(w, s[0])) || out(ldd4(w, s[1])) || out(ldd4(w, s[4])) || out(ldd4(w, s[5]));
         if (bad) return false;
     }
@@ -355,11 +363,8 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     const Roe2 C = roe2(W1, P1, gm1);
     if (GUARD && !(C.R.H.h - C.R.hq2.h >= 0.25f * C.R.H.h)) return false;
     {
-        f2 finite = pk(0.0f, 0.0f);  // 0 while every field is
         auto put = [&](const vec4<f2> &d, int slot) {
             const vec4<f2> c = project_n(C.R, d);
-            const f2 z = pk(0.0f, 0.0f);
-            if (GUARD) finite = ffma(c.x.h, z, ffma(c.n.h, z, ffma(c.t.h, z, ffma(c.w.h, z, finite))));
             st_dw2(S, slot, norm(c.x));
             st_dw2(S, slot + 1, norm(c.n));
             st_dw2(S, slot + 2, norm(c.t));
@@ -367,7 +372,6 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
         };
         put(dpair(s[1], s[4]), kSlotBF);
         put(dpair(s[0], s[5]), kSlotAE);
-        if (GUARD && !(lane0(finite) == 0.0f && lane1(finite) == 0.0f)) return false;
         const vec4<float> c = project_n(C.R, dmid());
         st_dw2(S, kSlotC, norm(pair(c.x, c.n)));
         st_dw2(S, kSlotC + 1, norm(pair(c.t, c.w)));
@@ -397,6 +401,8 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
         ok = lane0(P.p.h) > 0.0f && lane1(P.p.h) > 0.0f;
     }
     if (!ok) {  // positivity fallback: the end states
+        // not for differences beyond FP32's range, which leave a NaN in every state
+        if (GUARD && !(lane0(dd.w.h) - lane0(dd.w.h) == 0.0f && lane1(dd.w.h) - lane1(dd.w.h) == 0.0f)) return false;
         Wi = W1;
         P = P1;
         jump = dmid();
@@ -469,13 +475,15 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     }
     wb = norm4(wb);
     double *G = A.G;  // [6][ne][4]
+    float chk = 0.0f;  // 0 while every output is finite (else FP64 writes them all again)
     auto put = [&](int slot, dw x, dw n, dw t, dw v) {  // back to x-y components and to FP64, unscaled
         const dw2 m = norm(lfma(pair(lneg(ny), nx), both(t), lmul(pair(nx, ny), both(n))));
         auto to = [&](float h, float l) {
             const double v = f2d_scaled(h, kl) + f2d_scaled(l, kl);
-            const bool finite = (__float_as_uint(h) & 0x7f800000u) != 0x7f800000u;
-            return finite ? v : __hiloint2double(0x7ff80000, 0);
+            const bool odd = !GUARD && (__float_as_uint(h) & 0x7f800000u) == 0x7f800000u;
+            return odd ? __hiloint2double(0x7ff80000, 0) : v;
         };
+        if (GUARD) chk = fmaf(x.h, 0.0f, fmaf(lane0(m.h), 0.0f, fmaf(lane1(m.h), 0.0f, fmaf(v.h, 0.0f, chk))));
         double2 *q = reinterpret_cast<double2 *>(G + 4 * ((int64_t)slot * ne + e));
         q[0] = make_double2(to(x.h, x.l), to(lane0(m.h), lane0(m.l)));
         q[1] = make_double2(to(lane1(m.h), lane1(m.l)), to(v.h, v.l));
@@ -488,7 +496,7 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
         put(3, second(wb.x), second(wb.n), second(wb.t), second(wb.w));
         put(4, z, z, z, z);
         put(5, z, z, z, z);
-        return true;
+        return !GUARD || chk == 0.0f;
     }
     // both interpolated states are L1 plus an increment
     const dw z = dw_make(0.0f);
@@ -532,7 +540,7 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
     }
     put(2, first(g1.x), first(g1.n), first(g1.t), first(g1.w));
     put(3, second(g1.x), second(g1.n), second(g1.t), second(g1.w));
-    return true;
+    return !GUARD || chk == 0.0f;
 }
 
 // At most 200 registers, 5 blocks (10 warps) per SM: 0.270 ms for the residual

@@ -137,11 +137,16 @@ __device__ __forceinline__ void clear_wide(const EdgeArgs &A, int64_t e) {
 
 // Writes the increment of edge e and returns true.  With GUARD (precision 64)
 // it returns false, writing nothing, where the double words would lose more
-// than FP64 does: an average whose c^2 is a small difference, (H - q^2/2) < H/4
-// (Mach numbers above 3.9), costs the double words log2(H / (H - q^2/2)) of
-// their 48 bits (measured on the flux itself against extended precision: at
-// amplitude 0.3 over 48 vertices 3e-16 at Mach 1, 7e-16 at 3, 7e-15 at 10), so
-// the caller takes those edges in FP64.
+// than FP64 does, and the caller takes the edge in FP64:
+//  - an average whose c^2 is a small difference, (H - q^2/2) < H/4 (Mach numbers
+//    above sqrt(6 / (gamma - 1)), 3.9 for gamma = 1.4), costs the double words
+//    log2(H / (H - q^2/2)) of their 48 bits (measured on the flux itself against
+//    extended precision: at amplitude 0.3 over 48 vertices 3e-16 at Mach 1, 7e-16
+//    at 3, 7e-15 at 10);
+//  - a state thinner than L1/64 formed from L1 costs log2 of that ratio.  Residual
+//    against extended precision, FP64 / double words without this / with it, flow
+//    across density steps of 64, 256, 1024, 4096: 2.1e-14 / 3.7e-15 / 5e-15, 2.4e-14
+//    / 1.6e-14 / 1.2e-14, 2.6e-14 / 1.5e-13 / 1.7e-14, 4.5e-14 / 1.4e-12 / 4e-14.
 template <bool GUARD>
 __device__ __forceinline__ bool edge_flux_dw_body(const EdgeArgs &A, const int64_t e, const Stage &S) {
     const double *__restrict__ w = static_cast<const double *>(A.w);
@@ -253,6 +258,8 @@ __device__ __forceinline__ bool edge_flux_dw_body(const EdgeArgs &A, const int64
         sides();
         fell_back = true;
     }
+
+    if (GUARD && !(fminf(lane0(P.rho.h), lane1(P.rho.h)) >= 0.015625f * b.x.h)) return false;
 
     // flux increment F_n(w_L) - F_n(L1)
     const vec4<float> il{first(dd.x), first(dd.n), first(dd.t), first(dd.w)};
