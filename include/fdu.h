@@ -259,7 +259,9 @@ fdu_status fdu_batch_set_dt(fdu_mesh *batch, const double *dt, void *stream);
 /* n_steps SSP-RK3 steps of every mesh (FP64 state accumulation; the
  * residual at `precision`, 64, 48 or 32 as for fdu_residual; precision 48
  * runs a kernel of its own with its double-word staging in dynamic shared
- * memory).  FDU_ERR_TIMEOUT if a grid barrier's bounded wait ran out.  The
+ * memory).  At precision 64 each mesh takes the arithmetic it would take
+ * alone: one out of the double words' range does not send the others to FP64.
+ * FDU_ERR_TIMEOUT if a grid barrier's bounded wait ran out.  The
  * batch's state is then undefined: blocks that were still waiting may have
  * given up while the others went on with their part of that stage.  Every
  * later launch of the call finds the error flag set and returns without

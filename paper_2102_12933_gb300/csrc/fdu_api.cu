@@ -91,10 +91,11 @@ struct fdu_mesh {
                                              // [4] stage updates scaled by the positivity safeguard,
                                              // [5] first non-physical row of a state being set
     // adaptive stepping: (t, dt, nonphysical flag), then the step counter and
-    // the wide flags in the fourth to sixth words, all reset with the state
+    // the wide flags from the fourth word on, all reset with the state
     double *tstate = nullptr;
     unsigned long long *nsteps = nullptr;    // adaptive steps taken (in tstate's fourth word)
-    int *wide = nullptr;                     // [kWideSlots] (in tstate's fifth and sixth words)
+    int *wide = nullptr;                     // [wide_groups()][kWideSlots] (from tstate's fifth word on)
+    int wide_groups() const { return n_comp > 0 ? 1 + n_comp : 1; }
     bool wide_clean = false;                 // no launch has set or could have set a wide flag since they were zeroed
     bool f64_valid = false, f32_valid = false;              // F64[0] / (w32, F32[0]) describe wn
     cudaStream_t own_stream = nullptr;
@@ -385,7 +386,8 @@ fdu_status build_dw_tables(fdu_mesh *m) {
     return FDU_OK;
 }
 
-constexpr int kTState = 6;  // doubles of the tstate allocation
+// doubles of the tstate allocation
+int tstate_words(const fdu_mesh *m) { return 4 + m->wide_groups() * kWideSlots / 2; }
 
 // Pack host tables into device layouts.
 fdu_status upload_tables(fdu_mesh *m) {
@@ -515,9 +517,9 @@ fdu_status upload_tables(fdu_mesh *m) {
         const unsigned long long inf_bits = 0x7FF0000000000000ull;
         CK(cudaMemcpy(m->counters + 2, &inf_bits, sizeof inf_bits, cudaMemcpyHostToDevice));
     }
-    static_assert(kWideSlots * sizeof(int) <= 2 * sizeof(double), "the wide flags share tstate's allocation");
-    if ((st = m->alloc(m->tstate, kTState))) return st;
-    CK(cudaMemset(m->tstate, 0, kTState * sizeof(double)));
+    static_assert(kWideSlots * sizeof(int) == 2 * sizeof(double), "the wide flags share tstate's allocation");
+    if ((st = m->alloc(m->tstate, tstate_words(m)))) return st;
+    CK(cudaMemset(m->tstate, 0, tstate_words(m) * sizeof(double)));
     m->nsteps = reinterpret_cast<unsigned long long *>(m->tstate + 3);
     m->wide = reinterpret_cast<int *>(m->tstate + 4);
     CK(cudaMemset(m->wn, 0, 4 * nv * sizeof(double)));
@@ -553,6 +555,8 @@ EdgeArgs edge_args(fdu_mesh *m, int prec, const void *w) {
     if (fp64_state(prec)) {
         a.coefdw = m->coefdw;
         a.wide = m->wide;
+        a.wcomp = m->comp;
+        a.n_comp = m->n_comp;
         dw_split(m->opts.gamma - 1.0, a.dw_gm1);
         dw_split(0.1, a.dw_tenth);
         int ee = 0;
@@ -590,6 +594,7 @@ DivArgs div_args(fdu_mesh *m, int prec, int fin) {
         a.F = m->F64[fin]; a.r = m->r64;  // the double-word increments take r64's storage
         a.kind = prec == 48 ? kDivDw : m->dw64 ? kDivGuard : kDivPlain;
         a.wide = m->wide;
+        a.wcomp = m->comp;
         a.wide_in = fin;
         a.wide_out = (fin + 1) % 3;
     } else {
@@ -629,9 +634,9 @@ void timed(fdu_mesh *m, int kind, bool allowed, cudaStream_t s, F &&launch) {
 // launch) can have left some, so that they depend on the state alone.
 void ensure_fluxes(fdu_mesh *m, int prec, cudaStream_t s) {
     if (fp64_state(prec) && !m->f64_valid) {
-        if (!m->wide_clean) cudaMemsetAsync(m->wide, 0, kWideSlots * sizeof(int), s);
+        if (!m->wide_clean) cudaMemsetAsync(m->wide, 0, m->wide_groups() * kWideSlots * sizeof(int), s);
         m->wide_clean = false;
-        launch_vertex_flux_f64(m->wn, m->F64[0], m->nv, m->opts.gamma, s, m->Q64[0], m->wide, m->n_real);
+        launch_vertex_flux_f64(m->wn, m->F64[0], m->nv, m->opts.gamma, s, m->Q64[0], m->wide, m->n_real, m->comp);
         m->f64_valid = true;
     }
     if (prec == 32 && !m->f32_valid) {
@@ -1189,7 +1194,7 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
     if (!w) return set_err(FDU_ERR_ARG, "null state");
     cudaStream_t s = m->stream(stream);
     if (on_device) {
-        launch_permute_rows(w, m->wn, m->new2old, m->nv, true, s, m->tstate, kTState);
+        launch_permute_rows(w, m->wn, m->new2old, m->nv, true, s, m->tstate, tstate_words(m));
         CK_LAUNCH();
     } else {
         // one copy of the caller's rows (a DMA when they are pinned), checked
@@ -1205,7 +1210,7 @@ fdu_status fdu_set_state(fdu_mesh *m, const double *w, int on_device, void *stre
         CK(cudaStreamSynchronize(s));
         if (bad != none)
             return set_err(FDU_ERR_NONPHYSICAL, "state row " + std::to_string(bad) + " has rho <= 0 or a non-finite value");
-        launch_permute_rows(m->scratch, m->wn, m->new2old, m->nv, true, s, m->tstate, kTState);
+        launch_permute_rows(m->scratch, m->wn, m->new2old, m->nv, true, s, m->tstate, tstate_words(m));
         CK_LAUNCH();
     }
     if (m->n_ghost > 0) {

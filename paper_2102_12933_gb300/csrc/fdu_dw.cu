@@ -80,11 +80,11 @@ __global__ void coef_dw_kernel(const double *__restrict__ coef, float4 *__restri
 }
 
 // Accuracy check of the double-word primitives: inputs and outputs as
-// doubles (inputs split by d2dw, outputs recombined exactly by f2d).
+// doubles (inputs split by d2dw, outputs recombined exactly by dw2d).
 __global__ void dw_check_kernel(int op, const double *__restrict__ x, const double *__restrict__ y,
                                 double *__restrict__ z, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    auto out = [&](dw r) { z[i] = f2d(r.h) + f2d(r.l); };
+    auto out = [&](dw r) { z[i] = dw2d(r); };
     if (op == 7) {  // compensated dot product of 8 consecutive pairs
         if (i >= n / 8) return;
         dot2 A{0.0f, 0.0f};

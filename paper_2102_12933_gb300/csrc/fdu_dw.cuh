@@ -145,15 +145,18 @@ __device__ __forceinline__ dw d2dw(double d) {
     const float l = (m != 0u && le > 0) ? __uint_as_float(sgn | ((unsigned)le << 23) | (lb & 0x7fffffu)) : 0.0f;
     return dw_make(h, l);  // |l| < ulp(h): the truncated split, not renormalised
 }
-// float -> double, exact for normal floats (zero and subnormals -> 0; infinities
-// and NaN stay what they are)
+// float -> double, exact for finite normal floats (zero and subnormals -> 0)
 __device__ __forceinline__ double f2d(float x) {
     const unsigned b = __float_as_uint(x);
-    const unsigned e = (b >> 23) & 0xffu, d = e == 255u ? 2047u : e + 896u;
+    const unsigned e = (b >> 23) & 0xffu;
     if (e == 0u) return 0.0;
-    return __hiloint2double((int)((b & 0x80000000u) | (d << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
+    return __hiloint2double((int)((b & 0x80000000u) | ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
 }
-
+// a double word; a NaN where its high word is not finite
+__device__ __forceinline__ double dw2d(dw x) {
+    const double v = f2d(x.h) + f2d(x.l);
+    return fabsf(x.h) < INFINITY ? v : __longlong_as_double(0x7ff8000000000000ll);
+}
 
 // ------------------------------------------------------------------ packed pairs, lean forms
 // Two FP32 lanes in a 64-bit register pair, and the explicitly rounded

@@ -130,9 +130,10 @@ __device__ __forceinline__ dw2 ld_dw2(const Stage &T, int j) {
 // slot of the step's result, cleared in the third stage just before that stage
 // writes it: a caller may stop after the second stage and keep the start state.
 __device__ __forceinline__ void clear_wide(const EdgeArgs &A, int64_t e) {
-    if (!A.wide || e != 0) return;
-    if (A.wide_in == 0) A.wide[1] = A.wide[2] = 0;
-    if (A.wide_in == 2) A.wide[0] = 0;
+    if (!A.wide || e > A.n_comp) return;
+    int *f = A.wide + kWideSlots * e;  // e: all meshes of a batch, or the one mesh (0), and each of a batch's
+    if (A.wide_in == 0) f[1] = f[2] = 0;
+    if (A.wide_in == 2) f[0] = 0;
 }
 
 // Writes the increment of edge e and returns true.  With GUARD (precision 64)

@@ -138,14 +138,40 @@ __device__ __noinline__ void edge_flux_f64_cold(const EdgeArgs *A, const int64_t
     }
     st4(static_cast<double *>(A->r), e, f);
 }
-// One edge at precision 64.
-__device__ __forceinline__ void edge_flux_guard_body(const EdgeArgs &A, const int64_t e, const dwa::Stage &S,
-                                                     const bool wide) {
-    if (wide) edge_flux_f64_cold(&A, e, false);
-    else if (!dwa::edge_flux_dw_body<true>(A, e, S)) edge_flux_f64_cold(&A, e, true);
-}
 __device__ __forceinline__ bool stage_is_wide(const int *wide, int in) {
     return (__ldcg(wide + in) | __ldcg(wide + kWideGhost)) != 0;
+}
+// The flag of vertex v's mesh, where any mesh's is set (through L1: no launch
+// writes the slot that it reads).
+template <class Args>
+__device__ __forceinline__ bool mesh_is_wide(const Args &A, int64_t v) {
+    return __ldca(A.wide + kWideSlots * (1 + __ldg(A.wcomp + v)) + A.wide_in) != 0;
+}
+__device__ __forceinline__ void set_wide(int *wide, const int32_t *wcomp, int64_t v, int slot) {
+    wide[slot] = 1;
+    if (wcomp) wide[kWideSlots * (1 + __ldg(wcomp + v)) + slot] = 1;
+}
+// Which meshes' stages are out of the window.
+enum Wide { kNone, kAll, kSome };
+template <class Args>
+__device__ __forceinline__ Wide wide_stage(const Args &A) {
+    return !stage_is_wide(A.wide, A.wide_in) ? kNone : A.wcomp ? kSome : kAll;
+}
+// The same, telling whether all of a batch's are, which spares every edge and
+// vertex the look at its mesh's flag (6 meshes, 167k vertices, all outside: 1984
+// to 1885 us a step); every thread of the block calls it.
+__device__ __forceinline__ Wide wide_batch_stage(const EdgeArgs &A) {
+    Wide k = wide_stage(A);
+    if (k != kSome) return k;
+    int all = 1;
+    for (int c = threadIdx.x; c < A.n_comp; c += blockDim.x) all &= __ldcg(A.wide + kWideSlots * (1 + c) + A.wide_in);
+    return __syncthreads_and(all) ? kAll : kSome;
+}
+// One edge at precision 64.
+__device__ __forceinline__ void edge_flux_guard_body(const EdgeArgs &A, const int64_t e, const dwa::Stage &S,
+                                                     const Wide k) {
+    if (k == kAll || (k == kSome && mesh_is_wide(A, __ldg(A.sten + 2 * A.ne + e)))) edge_flux_f64_cold(&A, e, false);
+    else if (!dwa::edge_flux_dw_body<true>(A, e, S)) edge_flux_f64_cold(&A, e, true);
 }
 // A state outside the double words' window: density or energy not in
 // [2^-kWideExp, 2^kWideExp), by the exponent field (NaN, zero, negative and
@@ -172,7 +198,7 @@ __device__ __forceinline__ dbl4 roe_record64(const dbl4 &w, const Prim64 &P) {
 }
 
 __global__ void vertex_flux_f64_kernel(const double *__restrict__ w, double *__restrict__ F, double *__restrict__ Q,
-                                       int64_t n, double gm1, int *wide, int64_t n_real) {
+                                       int64_t n, double gm1, int *wide, int64_t n_real, const int32_t *wcomp) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
     const dbl4 s = ld4(w, v);
@@ -182,7 +208,7 @@ __global__ void vertex_flux_f64_kernel(const double *__restrict__ w, double *__r
     st4(F, 2 * v, f);
     st4(F, 2 * v + 1, g);
     if (Q) st4(Q, v, roe_record64(s, P));
-    if (wide && outside_window(s, P.p)) wide[v < n_real ? 0 : kWideGhost] = 1;
+    if (wide && outside_window(s, P.p)) set_wide(wide, wcomp, v, v < n_real ? 0 : kWideGhost);
 }
 
 // Forward-Euler part of an SSP-RK3 stage, fe = ws + theta dt L.  Without
@@ -300,10 +326,10 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i, 
             dot2_add(sw, a, dw_make(q1.z, q1.w));
         }
         const dw rx = dot2_result(sx), ry = dot2_result(sy), rz = dot2_result(sz), rw = dot2_result(sw);
-        acc.x += f2d(rx.h) + f2d(rx.l);
-        acc.y += f2d(ry.h) + f2d(ry.l);
-        acc.z += f2d(rz.h) + f2d(rz.l);
-        acc.w += f2d(rw.h) + f2d(rw.l);
+        acc.x += dw2d(rx);
+        acc.y += dw2d(ry);
+        acc.z += dw2d(rz);
+        acc.w += dw2d(rw);
     } else {
         const int64_t b = __ldg(A.slice_eoff + sl) + lane, e = on ? __ldg(A.slice_eoff + sl + 1) : 0;
 #pragma unroll 4
@@ -365,7 +391,7 @@ __device__ __forceinline__ void div_f64_body(const DivArgs &A, const int64_t i, 
     st4(Fo, 2 * v, f);
     st4(Fo, 2 * v + 1, g);
     if (A.Qout) st4(A.Qout, v, roe_record64(o, P));
-    if (A.wide && outside_window(o, P.p)) A.wide[A.wide_out] = 1;
+    if (A.wide && outside_window(o, P.p)) set_wide(A.wide, A.wcomp, v, A.wide_out);
 }
 // The FP64 form out of line, for the kernels that seldom take it.  It shares a
 // vertex between the same lanes: RK3 step outside the window with one of them at
@@ -377,17 +403,19 @@ template <int MODE, int LPV>
 __device__ __noinline__ void div_f64_cold(const DivArgs *A, const int64_t i, const int q, const bool on) {
     div_f64_body<MODE, false, LPV>(*A, i, q, on);
 }
-// The divergence of one vertex by KIND (kDivPlain, kDivDw, kDivGuard).
+// The divergence of one vertex by KIND (kDivPlain, kDivDw, kDivGuard).  Lanes that
+// share a warp but not a mesh take one form after the other, each with the
+// other's lanes off.
 template <int MODE, int KIND, int LPV = 1>
-__device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, const bool wide, const int q = 0,
-                                            const bool on = true) {
-    if (KIND == kDivPlain) {
-        div_f64_body<MODE, false, LPV>(A, i, q, on);
-    } else if (KIND == kDivGuard && wide) {
-        div_f64_cold<MODE, LPV>(&A, i, q, on);
-    } else {
-        div_f64_body<MODE, true, LPV>(A, i, q, on);
+__device__ __forceinline__ void div_f64_any(const DivArgs &A, const int64_t i, const Wide k, const int q = 0,
+                                            bool on = true) {
+    if (KIND == kDivGuard && k != kNone) {
+        const bool wide = on && (k == kAll || mesh_is_wide(A, A.perm ? (int64_t)__ldg(A.perm + i) : i));
+        if (LPV == 1 ? wide : __any_sync(0xffffffffu, wide)) div_f64_cold<MODE, LPV>(&A, i, q, wide);
+        on = on && !wide;
+        if (LPV == 1 ? !on : !__any_sync(0xffffffffu, on)) return;
     }
+    div_f64_body<MODE, KIND != kDivPlain, LPV>(A, i, q, on);
 }
 
 // ================================================================== FP32 path
@@ -807,7 +835,7 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) edge_flux_guard_kernel(const __
     if (e >= A.ne) return;
     if (A.dt_dev && *A.dt_dev == 0.0) return;
     dwa::clear_wide(A, e);
-    edge_flux_guard_body(A, e, dwa::Stage{stage + threadIdx.x, kEdgeBlock}, stage_is_wide(A.wide, A.wide_in));
+    edge_flux_guard_body(A, e, dwa::Stage{stage + threadIdx.x, kEdgeBlock}, wide_stage(A));
 }
 // At most 80 registers (6 blocks, 24 warps per SM): with the 56 the compiler
 // takes when left alone fewer gathers are in flight (precision 48 0.139 against
@@ -817,7 +845,7 @@ __global__ void __launch_bounds__(kDivBlock, 6) div_f64_kernel(const __grid_cons
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LPV;
     if (LPV == 1 && i >= A.n_real) return;
     if (MODE != 0 && A.dt_dev && *A.dt_dev == 0.0) return;  // adaptive run already at t_end
-    div_f64_any<MODE, KIND, LPV>(A, i, KIND == kDivGuard && stage_is_wide(A.wide, A.wide_in),
+    div_f64_any<MODE, KIND, LPV>(A, i, KIND == kDivGuard ? wide_stage(A) : kNone,
                                  (int)threadIdx.x % LPV, i < A.n_real);
 }
 // ------------------------------------------------------------------ divergence tiles
@@ -1330,9 +1358,9 @@ __global__ void __launch_bounds__(512, 1)
     const dwa::Stage T{dw_stage + threadIdx.x, (int)blockDim.x};
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool wide = GUARD && stage_is_wide(EA.wide, EA.wide_in);
+    const Wide wide = GUARD ? wide_batch_stage(EA) : kNone;
+    for (int64_t c = t0; c <= EA.n_comp; c += stride) dwa::clear_wide(EA, c);
     for (int64_t e = t0; e < EA.ne; e += stride) {
-        dwa::clear_wide(EA, e);
         if (GUARD) edge_flux_guard_body(EA, e, T, wide);
         else dwa::edge_flux_dw_body<false>(EA, e, T);
     }
@@ -1528,8 +1556,8 @@ inline unsigned blocks(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 }  // namespace
 
 void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q, int *wide,
-                            int64_t n_real) {
-    if (n > 0) vertex_flux_f64_kernel<<<blocks(n, 256), 256, 0, s>>>(w, F, Q, n, gamma - 1.0, wide, n_real);
+                            int64_t n_real, const int32_t *wcomp) {
+    if (n > 0) vertex_flux_f64_kernel<<<blocks(n, 256), 256, 0, s>>>(w, F, Q, n, gamma - 1.0, wide, n_real, wcomp);
 }
 void launch_fold_tables(const DivArgs &a, const int32_t *left, const double *nx, const double *ny, double *wf48,
                         double *wg48, float2 *we48, double *cfg48, int *bad, cudaStream_t s) {

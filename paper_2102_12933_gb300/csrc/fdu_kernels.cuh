@@ -20,7 +20,10 @@ constexpr int kDivBlock = 128;   // threads per block, divergence kernels
 // that finds wide[in] or wide[3] set runs in FP64 throughout.  The edge kernels
 // clear the slots (clear_wide): the first stage's those of the two intermediate
 // states, the third stage's that of the result, so that the flag of a state
-// whose step is only partly taken (the adjoint's recomputation) stands.
+// whose step is only partly taken (the adjoint's recomputation) stands.  A batch
+// has a group of kWideSlots flags for each of its meshes after the first group,
+// which then says whether any mesh's is set: a mesh takes the arithmetic that it
+// would take alone.
 constexpr int kWideGhost = 3;
 constexpr int kWideSlots = 4;
 constexpr int kWideExp = 24;
@@ -53,6 +56,8 @@ struct EdgeArgs {
     // (WideFlags), and the buffer slot of the stage state; nullptr: FP64 only
     int *wide;
     int wide_in;
+    const int32_t *wcomp; // batch: mesh of each vertex (nullptr: one mesh)
+    int n_comp;           // and their number
 };
 
 
@@ -81,6 +86,7 @@ struct DivArgs {
     int kind;                    // FP64 state: kDivPlain, kDivDw or kDivGuard
     int *wide;                   // WideFlags (nullptr: not kept), and the slots of the stage's input and output
     int wide_in, wide_out;
+    const int32_t *wcomp;        // batch: mesh of each vertex, for the flags
     // residual output (mode 0)
     double *out;                 // [nv][4] FP64
     const int32_t *out_map;      // internal -> output row (nullptr = internal order)
@@ -137,9 +143,9 @@ void launch_tile_count(const TileSource &S, const TileTables &T, int32_t *nv, in
 void launch_tile_fill(const TileSource &S, const TileTables &T, cudaStream_t s);
 
 // F[v] = (f, g) of w[v]; Q (optional) = Roe records (sqrt rho, sqrt rho u, sqrt rho v, sqrt rho H)
-// wide (optional): slot 0 of the WideFlags for vertices below n_real, kWideGhost for the others
+// wide (optional): slot 0 of the WideFlags for vertices below n_real, kWideGhost for the others; wcomp: a batch's meshes
 void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma, cudaStream_t s, double *Q = nullptr,
-                            int *wide = nullptr, int64_t n_real = 0);
+                            int *wide = nullptr, int64_t n_real = 0, const int32_t *wcomp = nullptr);
 void launch_vertex_flux_f32(const double *w, float4 *F, float4 *w32, int64_t n, double gamma, cudaStream_t s);
 void launch_edge_flux_f64(const EdgeArgs &a, cudaStream_t s);    // FP64 throughout
 void launch_edge_flux_guard(const EdgeArgs &a, cudaStream_t s);  // precision 64: double words within the window
@@ -160,7 +166,7 @@ void launch_div_f32(const DivArgs &a, int mode, cudaStream_t s);
 void launch_div_f32_tiles(const DivArgs &a, const TileTables &t, int mode, cudaStream_t s);
 // *bad = min(*bad, first row of w[n][4] with rho <= 0 or a non-finite value)
 void launch_check_rows(const double *w, int64_t n, unsigned long long *bad, cudaStream_t s);
-// zero (optional): nzero (at most 256) doubles that the launch also sets to 0
+// zero (optional): nzero doubles (at most max(n, 256)) that the launch also sets to 0
 void launch_permute_rows(const double *in, double *out, const int32_t *map, int64_t n, bool gather, cudaStream_t s,
                          double *zero = nullptr, int nzero = 0);
 void launch_ghost_fill(double *w, const double *wsrc, void *F, const void *Fsrc, int fq, double *Q, const double *Qsrc,

@@ -61,3 +61,29 @@ def test_wide_state_over_the_lanes_of_a_vertex(n):
     M.rk_step(dt, 64)
     one = M.get_state()
     assert np.linalg.norm(wide - one) <= 1e-11 * np.linalg.norm(one - w)
+
+
+@pytest.mark.parametrize("sizes", [(16, 23, 29), (60, 90, 100), (150, 160, 170)])
+@pytest.mark.parametrize("spoilt", [0, 1, 2])
+def test_meshes_of_a_batch_keep_to_themselves(sizes, spoilt):
+    """One mesh of a batch outside the window (in density units of 2^40): it takes
+    the bits that it has when all of them are, and the others those that they
+    have when none is, in residuals (four, two and one lanes to a vertex) and in
+    persistent steps."""
+    cases = [inputs.vortex_case(n, seed=n, beta=3.0) for n in sizes]
+    B = fdu.Batch([(m.xy, m.tri) for m, _ in cases], L=10.0, weno_eps=1e-300)
+    s = 2.0 ** 40
+    scale = {"none": [1.0] * 3, "all": [s] * 3, "one": [s if i == spoilt else 1.0 for i in range(3)]}
+    out = {}
+    for k, f in scale.items():
+        B.set_state(np.concatenate([w * a for (_, w), a in zip(cases, f)]))
+        B.set_dt(B.batch_max_dt(0.4))
+        r = B.residual(64)
+        B.batch_rk_steps(2, 64)
+        p = B.get_state()
+        B.rk_step(1e-3, 64)
+        out[k] = (r, p, B.get_state())
+    for i in range(3):
+        rows = slice(B.offsets[i], B.offsets[i + 1])
+        for got, want in zip(out["one"], out["all" if i == spoilt else "none"]):
+            assert np.array_equal(got[rows], want[rows])
