@@ -91,7 +91,7 @@ typedef struct fdu_mesh_info {
     int64_t div_vert_nnz;    /* vertex entries over all divergence stencils */
     int64_t div_edge_nnz;    /* edge entries over all divergence stencils */
     int32_t J_min, J_max, K_min, K_max; /* stencil sizes (vertex, edge entries) */
-    int64_t device_bytes;    /* device memory held by the mesh */
+    int64_t device_bytes;    /* device memory held by the mesh (allocations, not what is used of them) */
     int64_t table_bytes_f64; /* bytes of the FP64 residual's read-only tables */
     int64_t table_bytes_f32; /* bytes of the FP32 residual's read-only tables */
     int32_t sell_width;      /* SELL slice width of the divergence tables */
@@ -118,6 +118,11 @@ fdu_status fdu_default_opts(fdu_mesh_opts *opts);
  * (the a1 and b2 rows of the pseudo-inverse); all in FP64 on the host,
  * then uploaded to the device unless opts->device = -1.
  *   xy[nv][2] FP64 vertex coordinates; tri[nt][3] int32 vertex ids.
+ * The device tables take about 5.4 KB per vertex, 2 of them for the faster
+ * kernels (double-word tables of precisions 64 and 48, tiles of precision 32).
+ * Where device memory has no room for those the mesh is created without them:
+ * precision 64 runs in FP64 throughout, precision 32 gathers from global
+ * memory, and precision 48 returns FDU_ERR_CUDA while there is no room.
  * Errors: FDU_ERR_ARG, FDU_ERR_MESH, FDU_ERR_STENCIL,
  * FDU_ERR_RANK_DEFICIENT, FDU_ERR_CUDA.  On error *out is NULL. */
 fdu_status fdu_mesh_create(const double *xy, int64_t nv, const int32_t *tri, int64_t nt, const fdu_mesh_opts *opts,

@@ -55,7 +55,7 @@ struct fdu_mesh {
     int device = -1;
     int64_t nv = 0, n_real = 0, n_ghost = 0, ne_act = 0, nslice = 0;
     int64_t vert_nnz_sell = 0, edge_nnz_sell = 0, vert_nnz_sell64 = 0, edge_nnz_sell64 = 0;
-    int64_t device_bytes = 0, table_bytes_f64 = 0, table_bytes_f32 = 0;
+    int64_t device_bytes = 0, table_bytes_f64 = 0, table_bytes_f32 = 0;  // device_bytes: allocated, chunks whole
     std::vector<void *> allocs;
     // tables
     int32_t *sten = nullptr;          // [6][ne_act]
@@ -68,8 +68,8 @@ struct fdu_mesh {
     double *swf48 = nullptr, *swg48 = nullptr, *cfg48 = nullptr;
     float2 *swe48 = nullptr;
     TileTables tile32{};              // FP32 divergence tiles (smem = 0: not used)
-    bool fold_ok = false;             // the folded tables hold (precision 48 is available)
-    bool dw64 = false;                // precision 64 takes the double-word path (fold_ok, tables in its window)
+    bool fold_ok = true;              // the tables fold (precision 48 is available; true until it is known)
+    bool dw64 = false;                // precision 64 takes the double-word path (tables held and in its window)
     int64_t *slice_voff = nullptr, *slice_eoff = nullptr;       // FP32 layout (natural order)
     int64_t *slice_voff64 = nullptr, *slice_eoff64 = nullptr;   // FP64 layout (stencil-size order in windows)
     int32_t *svid64 = nullptr, *seid64 = nullptr, *perm64 = nullptr;
@@ -142,32 +142,56 @@ struct fdu_mesh {
     static constexpr size_t kChunkMin = 4 << 20, kChunkMax = 64 << 20, kAlign = 256;
     char *chunk = nullptr;
     size_t chunk_left = 0;
+    bool no_memory = false;  // the last alloc that failed found no device memory
+    fdu_status device_alloc(void *&q, size_t bytes) {
+        const cudaError_t e = cudaMalloc(&q, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();  // not for the next launch check to find
+            no_memory = e == cudaErrorMemoryAllocation;
+            return set_err(FDU_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+        }
+        allocs.push_back(q);
+        device_bytes += (int64_t)bytes;
+        return FDU_OK;
+    }
     template <class T>
     fdu_status alloc(T *&p, size_t count) {
         p = nullptr;
         if (count == 0) count = 1;
         const size_t bytes = (count * sizeof(T) + kAlign - 1) / kAlign * kAlign;
-        const size_t next = std::clamp((size_t)device_bytes / 2 / kAlign * kAlign, kChunkMin, kChunkMax);
-        if (bytes > chunk_left || bytes > next / 4) {
-            void *q = nullptr;
-            const size_t take = bytes > next / 4 ? bytes : next;
-            cudaError_t e = cudaMalloc(&q, take);
-            if (e != cudaSuccess) return set_err(FDU_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-            allocs.push_back(q);
-            if (bytes > next / 4) {
-                device_bytes += (int64_t)(count * sizeof(T));
-                p = static_cast<T *>(q);
-                return FDU_OK;
-            }
+        const size_t held = (size_t)device_bytes - chunk_left;
+        const size_t next = std::clamp(held / 2 / kAlign * kAlign, kChunkMin, kChunkMax);
+        void *q = nullptr;
+        if (bytes > chunk_left && bytes <= next / 4 && device_alloc(q, next) == FDU_OK) {
             chunk = static_cast<char *>(q);
-            chunk_left = take;
+            chunk_left = next;
         }
-        void *q = chunk;
-        chunk += bytes;
-        chunk_left -= bytes;
-        device_bytes += (int64_t)(count * sizeof(T));
+        if (bytes > chunk_left || bytes > next / 4) {
+            if (fdu_status st = device_alloc(q, bytes)) return st;
+        } else {
+            q = chunk;
+            chunk += bytes;
+            chunk_left -= bytes;
+        }
         p = static_cast<T *>(q);
         return FDU_OK;
+    }
+    // A point that allocations can be taken back to.
+    struct Mark {
+        size_t n;
+        char *chunk;
+        size_t left;
+        int64_t bytes;
+    };
+    Mark mark() const { return Mark{allocs.size(), chunk, chunk_left, device_bytes}; }
+    void rewind(const Mark &k) {
+        while (allocs.size() > k.n) {
+            cudaFree(allocs.back());
+            allocs.pop_back();
+        }
+        chunk = k.chunk;
+        chunk_left = k.left;
+        device_bytes = k.bytes;
     }
     template <class T>
     fdu_status upload(T *&p, const std::vector<T> &h) {
@@ -274,22 +298,6 @@ void stencil_gaps(const double xi[6], float g[4]) {
     for (int c = 0; c < 4; ++c) g[c] = (float)d[c];
 }
 
-// The double-word tables of precisions 64 and 48, formed on the device from the
-// FP64 tables (on the host this took 0.2 s at 250k vertices, here a
-// millisecond):
-//  - the double-word edge coefficient block (hi = the FP32 rounding of each
-//    FP64 coefficient, lo = the FP32 rounding of the remainder);
-//  - divergence tables in the FP64 SELL layout where the edge flux, which
-//    the double-word edge kernel leaves as the increment
-//    r_k - F_n(L1_k) = r_k - (n_x f + n_y g)(L1_k), has its left-vertex part
-//    folded into the weights of that vertex's fluxes:
-//      sum_k w_k r_k = sum_k w_k (n_x,k f_L1k + n_y,k g_L1k) + sum_k w_k (r_k - F_n(L1_k)),
-//    the first sum going into w_f, w_g (or the centre weights when L1_k is
-//    the vertex itself) and the second taken in double words.
-//    Both ends of every stencil edge are in the vertex's own stencil, so
-//    the folding adds no entries; where that fails the mesh has no precision
-//    48, and precision 64 runs in FP64 throughout, as it does where a table
-//    entry or gamma - 1 is too large or small for the double words' range.
 // FP32 divergence tiles, formed on the device from the FP32 SELL tables: sizes
 // first (read back to place the lists), then lists, positions and weights.
 // T.smem stays 0, and the divergence gathers from global memory, where a tile
@@ -365,6 +373,22 @@ fdu_status build_tiles(fdu_mesh *m) {
 }
 
 DivArgs div_args(fdu_mesh *m, int prec, int fin);
+// The double-word tables of precisions 64 and 48, formed on the device from the
+// FP64 tables (on the host this took 0.2 s at 250k vertices, here a
+// millisecond):
+//  - the double-word edge coefficient block (hi = the FP32 rounding of each
+//    FP64 coefficient, lo = the FP32 rounding of the remainder);
+//  - divergence tables in the FP64 SELL layout where the edge flux, which
+//    the double-word edge kernel leaves as the increment
+//    r_k - F_n(L1_k) = r_k - (n_x f + n_y g)(L1_k), has its left-vertex part
+//    folded into the weights of that vertex's fluxes:
+//      sum_k w_k r_k = sum_k w_k (n_x,k f_L1k + n_y,k g_L1k) + sum_k w_k (r_k - F_n(L1_k)),
+//    the first sum going into w_f, w_g (or the centre weights when L1_k is
+//    the vertex itself) and the second taken in double words.
+//    Both ends of every stencil edge are in the vertex's own stencil, so
+//    the folding adds no entries; where that fails the mesh has no precision
+//    48, and precision 64 runs in FP64 throughout, as it does where a table
+//    entry or gamma - 1 is too large or small for the double words' range.
 fdu_status build_dw_tables(fdu_mesh *m) {
     const int64_t ne = m->ne_act, nr = std::max<int64_t>(m->n_real, 1);
     fdu_status st;
@@ -373,16 +397,41 @@ fdu_status build_dw_tables(fdu_mesh *m) {
     if ((st = m->alloc(m->swg48, m->vert_nnz_sell64))) return st;
     if ((st = m->alloc(m->swe48, m->edge_nnz_sell64))) return st;
     if ((st = m->alloc(m->cfg48, 2 * nr))) return st;
-    int bad = 0, *dbad = m->wide;  // zero here, and again below
+    int bad = 0, *dbad = reinterpret_cast<int *>(m->counters + 5);  // the row check's word, free between calls
+    CK(cudaMemset(dbad, 0, sizeof bad));
     launch_coef_dw(m->coef64, m->coefdw, ne, dbad, nullptr);
     launch_fold_tables(div_args(m, 64, 0), m->sten + 2 * ne, m->coef64 + (int64_t)kCoefN * ne,
                        m->coef64 + (int64_t)(kCoefN + 1) * ne, m->swf48, m->swg48, m->swe48, m->cfg48, dbad, nullptr);
     CK_LAUNCH();
     CK(cudaMemcpy(&bad, dbad, sizeof bad, cudaMemcpyDeviceToHost));
-    CK(cudaMemset(dbad, 0, sizeof bad));
     const double gm1 = m->opts.gamma - 1.0;
     m->fold_ok = (bad & 1) == 0;
     m->dw64 = bad == 0 && gm1 > 0x1p-10 && gm1 < 0x1p10;
+    return FDU_OK;
+}
+// The same, taken back where it failed or the tables do not fold.
+fdu_status try_dw_tables(fdu_mesh *m) {
+    const fdu_mesh::Mark k = m->mark();
+    m->no_memory = false;
+    const fdu_status st = build_dw_tables(m);
+    if (st || !m->fold_ok) {
+        m->coefdw = nullptr;
+        m->rewind(k);
+    }
+    return st;
+}
+// The tables of the faster kernels.  Where device memory has no room for them the
+// mesh does without: precision 64 then runs in FP64 throughout, precision 32
+// gathers from global memory, and precision 48 asks for its tables again at its
+// next use.
+fdu_status build_device_tables(fdu_mesh *m) {
+    fdu_status st = try_dw_tables(m);
+    if (st && !m->no_memory) return st;
+    const fdu_mesh::Mark k = m->mark();
+    m->no_memory = false;
+    st = build_tiles(m);
+    if (st && !m->no_memory) return st;
+    if (m->tile32.smem == 0) m->rewind(k);
     return FDU_OK;
 }
 
@@ -523,8 +572,7 @@ fdu_status upload_tables(fdu_mesh *m) {
     m->nsteps = reinterpret_cast<unsigned long long *>(m->tstate + 3);
     m->wide = reinterpret_cast<int *>(m->tstate + 4);
     CK(cudaMemset(m->wn, 0, 4 * nv * sizeof(double)));
-    if ((st = build_dw_tables(m))) return st;
-    return build_tiles(m);
+    return FDU_OK;
 }
 
 // Precision 48: the FP64 state pipeline (FP64 divergence and stage) with
@@ -534,6 +582,11 @@ inline int prof_kind(int prec) { return prec == 64 ? 0 : prec == 32 ? 2 : 4; }
 
 fdu_status check_precision(fdu_mesh *m, int prec) {
     if (prec != 64 && prec != 32 && prec != 48) return set_err(FDU_ERR_ARG, "precision must be 64, 48 or 32");
+    if (prec == 48 && m->fold_ok && !m->coefdw) {  // there was no memory for them
+        const fdu_status st = try_dw_tables(m);
+        m->dw64 = false;  // precision 64 stays as it was
+        if (st) return st;
+    }
     if (prec == 48 && !m->fold_ok)
         return set_err(FDU_ERR_MESH, "precision 48: an edge's left vertex is outside the vertex's stencil");
     return FDU_OK;
@@ -1087,6 +1140,7 @@ static fdu_status mesh_create(const double *xy, int64_t nv, const CellList &cell
             return set_err(FDU_ERR_CUDA, std::string("device setup: ") + cudaGetErrorString(e));
         }
         st = upload_tables(m);
+        if (st == FDU_OK) st = build_device_tables(m);
         if (st != FDU_OK) {
             std::string keep = g_err;
             m->release();
@@ -1484,6 +1538,7 @@ fdu_status fdu_batch_create(int32_t n_meshes, const double *const *xy, const int
     if (st == FDU_OK) st = m->alloc(m->comp_slots, n_meshes);
     if (st == FDU_OK) st = m->alloc(m->bar, 2);
     if (st == FDU_OK) st = m->alloc(m->bar_err, 1);
+    if (st == FDU_OK) st = build_device_tables(m);
     if (st == FDU_OK) {
         cudaMemset(m->dt_comp, 0, n_meshes * sizeof(double));
         cudaMemset(m->bar, 0, 2 * sizeof(unsigned int));
