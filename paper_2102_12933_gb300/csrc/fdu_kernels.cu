@@ -1188,55 +1188,66 @@ __global__ void __launch_bounds__(kTile, 7) div_f32_tile_kernel(const __grid_con
     div_f32_tile_body<MODE>(A, T, blockIdx.x, threadIdx.x, sm, [] { __syncthreads(); });
 }
 
-// Folded tables of the double-word divergence (launch_fold_tables); thread i
-// serves SELL position i.  Entries and sums in the order of the SELL lists,
-// rounded one by one.
+// Folded tables of the double-word divergence (launch_fold_tables).  Entries and
+// sums in the order of the SELL lists, rounded one by one.  kFoldLanes threads
+// serve a SELL position: each takes every kFoldLanes-th vertex entry, sums in
+// registers the edges whose left vertex it is, and looks at all of the position's
+// edges for that (independent loads).  One thread per position, adding to the
+// table for each edge in turn, waited for its own stores: the double-word tables
+// of 1600 vertices took 172 us in all, 118 now.
+constexpr int kFoldLanes = 8;
 __global__ void fold_tables_kernel(DivArgs A, const int32_t *__restrict__ left, const double *__restrict__ nx,
                                    const double *__restrict__ ny, double *wf48, double *wg48, float2 *we48,
                                    double *cfg48, int *bad) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kFoldLanes;
+    const int sub = (int)threadIdx.x % kFoldLanes;
     const int64_t sl = i / kSell;
-    if (sl >= (A.n_real + kSell - 1) / kSell) return;
+    if (sl >= (A.n_real + kSell - 1) / kSell) return;  // a slice's threads fill whole warps
     const int lane = (int)(i % kSell);
     const int64_t vb = A.slice_voff[sl] + lane, ve = A.slice_voff[sl + 1];
     const int64_t eb = A.slice_eoff[sl] + lane, ee = A.slice_eoff[sl + 1];
-    const double *wf = static_cast<const double *>(A.wf), *wg = static_cast<const double *>(A.wg);
-    const double *we = static_cast<const double *>(A.we), *cfg = static_cast<const double *>(A.cfg);
-    int flag = 0;
-    for (int64_t p = vb; p < ve; p += kSell) {
-        wf48[p] = wf[p];
-        wg48[p] = wg[p];
-        if (!(fabs(wf[p]) < kDwMax && fabs(wg[p]) < kDwMax)) flag |= 2;
-    }
+    const double *__restrict__ wf = static_cast<const double *>(A.wf), *__restrict__ wg = static_cast<const double *>(A.wg);
+    const double *__restrict__ we = static_cast<const double *>(A.we), *__restrict__ cfg = static_cast<const double *>(A.cfg);
     const bool real = i < A.n_real;
-    const int32_t v = real ? A.perm[i] : 0;
-    double cf = real ? cfg[v] : 0.0, cg = real ? cfg[A.n_real + v] : 0.0;
-    for (int64_t q = eb; q < ee; q += kSell) {
+    const int32_t v = real ? A.perm[i] : -1;
+    int flag = 0, edges = 0, found = 0;
+    // f, g += the normals of the edges (not padding) that start at `id`, times their weights
+    auto sum = [&](int32_t id, double &f, double &g) {
+#pragma unroll 4
+        for (int64_t q = eb; q < ee; q += kSell) {
+            const double w = we[q];
+            const int32_t e = A.eid[q];
+            if (w == 0.0 || left[e] != id) continue;
+            f = __dadd_rn(f, __dmul_rn(w, nx[e]));
+            g = __dadd_rn(g, __dmul_rn(w, ny[e]));
+            ++found;
+        }
+    };
+    for (int64_t p = vb + (int64_t)kSell * sub; p < ve; p += kSell * kFoldLanes) {
+        double f = wf[p], g = wg[p];
+        if (!(fabs(f) < kDwMax && fabs(g) < kDwMax)) flag |= 2;
+        const int32_t id = A.vid[p];
+        if (id != v) sum(id, f, g);  // padding names v itself
+        wf48[p] = f;
+        wg48[p] = g;
+    }
+    for (int64_t q = eb + (int64_t)kSell * sub; q < ee; q += kSell * kFoldLanes) {
         const double w = we[q];
         const float h = __double2float_rn(w);
         we48[q] = make_float2(h, __double2float_rn(w - (double)h));
         if (!(fabs(w) < kDwMax)) flag |= 2;
-        if (w == 0.0) continue;  // padding
-        const int32_t e = A.eid[q], L = left[e];
-        const double ax = __dmul_rn(w, nx[e]), ay = __dmul_rn(w, ny[e]);
-        if (L == v) {
-            cf = __dadd_rn(cf, ax);
-            cg = __dadd_rn(cg, ay);
-            continue;
-        }
-        int64_t p = vb;
-        while (p < ve && A.vid[p] != L) p += kSell;
-        if (p >= ve) {
-            flag |= 1;
-            continue;
-        }
-        wf48[p] = __dadd_rn(wf48[p], ax);
-        wg48[p] = __dadd_rn(wg48[p], ay);
+        edges += w != 0.0;
     }
-    if (real) {
-        cfg48[v] = cf;
-        cfg48[A.n_real + v] = cg;
+    if (real && sub == kFoldLanes - 1) {
+        double f = cfg[v], g = cfg[A.n_real + v];
+        sum(v, f, g);
+        cfg48[v] = f;
+        cfg48[A.n_real + v] = g;
     }
+    // every edge belongs to one entry or to the centre
+    int miss = edges - found;
+    for (int o = 1; o < kFoldLanes; o <<= 1) miss += __shfl_xor_sync(0xffffffffu, miss, o);
+    if (real && miss != 0) flag |= 1;
     if (flag) atomicOr(bad, flag);
 }
 template <int MODE>
@@ -1562,7 +1573,7 @@ void launch_vertex_flux_f64(const double *w, double *F, int64_t n, double gamma,
 void launch_fold_tables(const DivArgs &a, const int32_t *left, const double *nx, const double *ny, double *wf48,
                         double *wg48, float2 *we48, double *cfg48, int *bad, cudaStream_t s) {
     if (a.n_real <= 0) return;
-    const int64_t n = (a.n_real + kSell - 1) / kSell * kSell;
+    const int64_t n = (a.n_real + kSell - 1) / kSell * kSell * kFoldLanes;
     fold_tables_kernel<<<blocks(n, 128), 128, 0, s>>>(a, left, nx, ny, wf48, wg48, we48, cfg48, bad);
 }
 void launch_vertex_flux_f32(const double *w, float4 *F, float4 *w32, int64_t n, double gamma, cudaStream_t s) {
