@@ -420,7 +420,11 @@ fdu_status fdu_check_weno_coef32(int device, const double *xi, double *k, int64_
  * 0 the split of x, 1 x + y (accurate sum), 2 x + y (sloppy sum), 3 x * y,
  * 4 x * y before renormalisation, 5 1/x, 6 1/sqrt(x) (x > 0 normal), 7 the
  * compensated dot product of each 8 consecutive pairs (n a multiple of 8;
- * z[n/8]).  FDU_ERR_ARG for a bad op or size. */
+ * z[n/8]).  The edge kernels' lean forms, n even, c = the y of the row's
+ * neighbour (row i xor 1): 8 x + y, 9 x * y, 10 x * y + c, 11 (x + c) * y + c,
+ * 12 1/x, 13 1/sqrt(x), 14 the high word of x + y normalised; 16..22 and
+ * 24..30 the same in the first and second lane of packed instructions, the
+ * neighbour's operands in the other.  FDU_ERR_ARG for a bad op or size. */
 fdu_status fdu_check_dw(int device, int op, const double *x, const double *y, double *z, int64_t n);
 
 /* Measurement helper with no counterpart in the paper: the FMA throughput

@@ -2004,7 +2004,8 @@ fdu_status fdu_set_adjoint_precision(fdu_mesh *m, int precision) {
 }
 
 fdu_status fdu_check_dw(int device, int op, const double *x, const double *y, double *z, int64_t n) {
-    if (!x || !y || !z || n < 0 || op < 0 || op > 7 || (op == 7 && n % 8 != 0))
+    if (!x || !y || !z || n < 0 || op < 0 || op > 30 || (op >= 8 && (op % 8 == 7 || n % 2 != 0)) ||
+        (op == 7 && n % 8 != 0))
         return set_err(FDU_ERR_ARG, "bad arguments");
     if (n == 0) return FDU_OK;
     CK(cudaSetDevice(device));

@@ -79,8 +79,84 @@ __global__ void coef_dw_kernel(const double *__restrict__ coef, float4 *__restri
     }
 }
 
-// Accuracy check of the double-word primitives: inputs and outputs as
-// doubles (inputs split by d2dw, outputs recombined exactly by dw2d).
+// The normalised algorithms, for the accuracy check alone (operations 1 to 6), as
+// analysed by Joldes, Muller and Popescu, "Tight and rigorous error bounds for
+// basic building blocks of double-word arithmetic", ACM TOMS 44(2), 2017:
+//   add      accurate sum (their Algorithm 6): relative error <= 3u^2
+//   add_sl   sloppy sum (Algorithm 5): absolute error about u^2 (|x| + |y|)
+//   mul      double-word product (Algorithm 11): relative error <= 5u^2
+//   mul_u    the same before its final Fast2Sum, for operands of a sum
+// with u = 2^-24.  The reciprocal and the reciprocal square root take the
+// FP32 hardware approximation (PTX rcp.approx / rsqrt.approx, relative error
+// below 2^-22) and one correction of second order in its residual e:
+//   1/x       = r (1 + e + e^2 + ...),      e = 1 - x r
+//   1/sqrt(x) = y (1 + e/2 + 3e^2/8 + ...), e = 1 - x y^2
+// leaving O(e^3) < 2^-60 besides the double-word rounding.
+// s + t = a + b exactly, for |a| >= |b| (or a = 0)
+__device__ __forceinline__ dw fast_two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b);
+    return dw{s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ dw add(dw x, dw y) {
+    const dw s = two_sum(x.h, y.h);
+    const dw t = two_sum(x.l, y.l);
+    const dw v = fast_two_sum(s.h, __fadd_rn(s.l, t.h));
+    return fast_two_sum(v.h, __fadd_rn(t.l, v.l));
+}
+__device__ __forceinline__ dw add_sl(dw x, dw y) {
+    const dw s = two_sum(x.h, y.h);
+    return fast_two_sum(s.h, __fadd_rn(s.l, __fadd_rn(x.l, y.l)));
+}
+__device__ __forceinline__ dw mul(dw x, dw y) {
+    const float ch = __fmul_rn(x.h, y.h);
+    const float cl1 = __fmaf_rn(x.h, y.h, -ch);
+    const float cl2 = __fmaf_rn(x.l, y.h, __fmul_rn(x.h, y.l));
+    return fast_two_sum(ch, __fadd_rn(cl1, cl2));
+}
+// The same product without the final renormalisation (|l| may reach about
+// 2 ulp(h)): for operands of a sum, which renormalises.
+__device__ __forceinline__ dw mul_u(dw x, dw y) {
+    const float ch = __fmul_rn(x.h, y.h);
+    const float cl1 = __fmaf_rn(x.h, y.h, -ch);
+    return dw{ch, __fadd_rn(cl1, __fmaf_rn(x.l, y.h, __fmul_rn(x.h, y.l)))};
+}
+__device__ __forceinline__ dw recip(dw x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x.h));
+    const float p = __fmul_rn(x.h, r);
+    const float ep = __fmaf_rn(x.h, r, -p);  // x.h r = p + ep exactly; 1 - p is exact (p near 1)
+    const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.0f, p), ep), __fmul_rn(x.l, r));
+    return fast_two_sum(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+}
+__device__ __forceinline__ dw rsqrt(dw x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x.h));
+    const float y2 = __fmul_rn(y, y);
+    const float y2l = __fmaf_rn(y, y, -y2);  // y^2 = y2 + y2l exactly
+    const float p = __fmul_rn(x.h, y2);
+    const float ep = __fmaf_rn(x.h, y2, -p);  // x.h y2 = p + ep exactly
+    const float e = __fsub_rn(__fsub_rn(1.0f, p), __fadd_rn(ep, __fmaf_rn(x.h, y2l, __fmul_rn(x.l, y2))));
+    return fast_two_sum(y, __fmul_rn(__fmul_rn(y, e), __fmaf_rn(0.375f, e, 0.5f)));
+}
+
+// The lean forms on one lane (float) or two (f2): operation k of a, b and c.
+template <class T>
+__device__ dwv<T> lean_op(int k, dwv<T> a, dwv<T> b, dwv<T> c) {
+    switch (k) {
+        case 0: return ladd(a, b);
+        case 1: return lmul(a, b);
+        case 2: return lfma(a, b, c);
+        case 3: return lfma(ladd(a, c), b, c);  // an operand that is not normalised
+        case 4: return lrecip(a);
+        case 5: return lrsqrt(a);
+        default: {
+            const dwv<T> r = norm(ladd(a, b));
+            return dwv<T>{r.h, fsub(r.h, r.h)};
+        }
+    }
+}
+// Accuracy check: inputs and outputs as doubles (inputs split by d2dw, outputs
+// recombined exactly by dw2d).
 __global__ void dw_check_kernel(int op, const double *__restrict__ x, const double *__restrict__ y,
                                 double *__restrict__ z, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -94,6 +170,14 @@ __global__ void dw_check_kernel(int op, const double *__restrict__ x, const doub
     }
     if (i >= n) return;
     const dw a = d2dw(x[i]), b = d2dw(y[i]);
+    if (op >= 8) {  // 8 + k alone; 16 + k and 24 + k in lane 0 and 1, the neighbour's operands in the other
+        const int64_t j = i ^ 1;
+        const dw a1 = d2dw(x[j]), b1 = d2dw(y[j]);
+        if (op < 16) out(lean_op(op - 8, a, b, b1));
+        else if (op < 24) out(first(lean_op(op - 16, pair(a, a1), pair(b, b1), pair(b1, b))));
+        else out(second(lean_op(op - 24, pair(a1, a), pair(b1, b), pair(b, b1))));
+        return;
+    }
     switch (op) {
         case 0: out(a); break;
         case 1: out(add(a, b)); break;

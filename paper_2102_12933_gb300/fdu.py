@@ -234,6 +234,9 @@ def check_weno_coef32(xi, device=0):
 
 DW_OPS = {"split": 0, "add": 1, "add_sloppy": 2, "mul": 3, "mul_unnormalised": 4, "recip": 5, "rsqrt": 6,
           "dot8": 7}
+# the lean forms alone and in either lane of the packed instructions
+for _k, _op in enumerate(["lean_add", "lean_mul", "lean_fma", "lean_chain", "lean_recip", "lean_rsqrt", "lean_high"]):
+    DW_OPS.update({_op: 8 + _k, _op + ".0": 16 + _k, _op + ".1": 24 + _k})
 
 
 def check_dw(op, x, y=None, device=0):
