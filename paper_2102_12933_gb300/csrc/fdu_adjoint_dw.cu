@@ -290,8 +290,9 @@ __device__ __forceinline__ double scaled_down(double x, int k) {
 // differences that are not finite in FP32 (a NaN or huge momentum), an average whose c^2 is a
 // small difference (edge_flux_dw_body), a cotangent that is not finite, or a
 // WENO epsilon so far below the state's squares that the derivative of the
-// weights rests on the rounding of the differences (eps < 2^-76 E^2: noise of
-// 2^-53 of the state, squared, would pass for an indicator), or end states more
+// weights rests on the rounding of the differences (eps < 2^-76 max(rho, E)^2:
+// noise of 2^-53 of the state, squared, would pass for an indicator; the fields
+// are in units of density and momentum, |m|^2 < 2 rho E), or end states more
 // than a factor of two apart in density or energy.  VJP against central
 // differences in extended precision, FP64 / double words without the last line /
 // with it, steps of 4, 16, 64 in density and pressure: 7.7e-14 / 1.4e-13 / 3.1e-14,
@@ -327,7 +328,7 @@ __device__ __forceinline__ bool edge_vjp_dw_body(const AdjEdgeArgs &A, const int
         auto hi = [](double x) { return (unsigned)__double2hiint(x); };
         auto out = [&](const d4v &q) { return hi(q.x) - lo >= n || hi(q.w) - lo >= n; };
         auto jump = [&](double a, double b) { return hi(a) - hi(b) + (1u << 20) > 1u << 21; };
-        bool bad = out(L1d) || out(R1d) || dexp(A.eps) < 2 * dexp(L1d.w) - 1023 - 76;
+        bool bad = out(L1d) || out(R1d) || dexp(A.eps) < 2 * max(dexp(L1d.x), dexp(L1d.w)) - 1023 - 76;
         bad = bad || jump(L1d.x, R1d.x) || jump(L1d.w, R1d.w);
         bad = bad || out(ldd4(w, s[0])) || out(ldd4(w, s[1])) || out(ldd4(w, s[4])) || out(ldd4(w, s[5]));
         if (bad) return false;

@@ -945,7 +945,7 @@ void enqueue_residual_vjp(fdu_mesh *m, const double *w, const double *lam, doubl
     ea.eps = m->opts.weno_eps;
     ea.prec = m->adj_prec;
     // precision 64: double words where the WENO epsilon can reach the guard's
-    // 2^-76 E^2 for energies of their window (2^-24 and up), FP64 otherwise
+    // 2^-76 max(rho, E)^2 for states of their window (2^-24 and up), FP64 otherwise
     ea.guard = m->adj_prec == 64 && m->dw64 && m->opts.weno_eps >= 0x1p-124;
     if (ea.guard) {
         ea.list = m->adj_list;

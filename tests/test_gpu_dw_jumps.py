@@ -51,3 +51,25 @@ def test_vjp_across_steps(ratio):
         M.set_state(w * s)
         out.append(M.residual_vjp(lam))
     assert _rel(out[0], out[1]) <= 2e-13
+
+
+@pytest.mark.parametrize("k,e", [(0, -60), (10, -90), (10, -100), (10, -110), (20, -110), (-10, -60), (-10, -100)])
+def test_vjp_with_an_epsilon_below_the_noise_of_the_state(k, e):
+    """A state with rounding noise, in units of density 2^k and velocity 2^-k, with
+    epsilon = 2^e of the density squared: where noise (2^-106 of it) would pass
+    for an indicator the derivative is FP64's, whatever the units.  Tolerance:
+    the adjoint's bound 1e-10."""
+    m = inputs.torus_lattice(32, seed=4)
+    rng = np.random.default_rng(1)
+    bump = 1 + 0.3 * np.exp(-4 * ((m.xy - 5) ** 2).sum(1))
+    w = inputs.primitive_to_conservative(bump, 0.7 + 0 * bump, 0.3 + 0 * bump, bump / 1.4)
+    w = w * (1 + 2.0 ** -52 * rng.integers(-3, 4, w.shape))
+    lam = rng.standard_normal(w.shape)
+    rho, vel = 2.0 ** k, 2.0 ** -k
+    unit = np.array([rho, rho * vel, rho * vel, rho * vel * vel])
+    out = []
+    for s in (1.0, 2.0 ** 40):
+        M = fdu.Mesh(m.xy, m.tri, m.Lx, m.Ly, weno_eps=rho * rho * s * s * 2.0 ** e)
+        M.set_state(w * unit * s)
+        out.append(M.residual_vjp(lam / unit) * unit)
+    assert _rel(out[0], out[1]) <= 1e-10
