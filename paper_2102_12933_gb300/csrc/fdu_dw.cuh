@@ -58,13 +58,15 @@ __device__ __forceinline__ dw dot2_result(const dot2 &A) { return two_sum(A.s, A
 // word the next 24 of the remaining 29 (relative error below 2^-47).  The
 // pair is not renormalised (|l| < ulp(h) instead of ulp(h)/2): the
 // operations that take it renormalise their results.  Magnitudes of 2^128 and
-// above, infinities and NaN give an infinity or a NaN.
+// above, infinities and NaN give an infinity or a NaN; BOUNDED leaves the test
+// for them out, where the caller's values are known to be finite and smaller.
+template <bool BOUNDED = false>
 __device__ __forceinline__ dw d2dw(double d) {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
     const int e = (int)((hi >> 20) & 0x7ffu);
     if (e <= 896) return dw_make(0.0f, 0.0f);
     const unsigned sgn = hi & 0x80000000u;
-    const float h = __uint_as_float(sgn | ((unsigned)min(e - 896, 255) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    const float h = __uint_as_float(sgn | ((unsigned)(BOUNDED ? e - 896 : min(e - 896, 255)) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
     const unsigned m = lo & 0x1fffffffu;  // value m 2^(e - 1075)
     const unsigned lb = __float_as_uint(__uint2float_rn(m));
     const int le = (int)((lb >> 23) & 0xffu) + (e - 1075);

@@ -137,8 +137,9 @@ __device__ __forceinline__ void clear_wide(const EdgeArgs &A, int64_t e) {
 }
 
 // Writes the increment of edge e and returns true.  With GUARD (precision 64)
-// it returns false, writing nothing, where the double words would lose more
-// than FP64 does, and the caller takes the edge in FP64:
+// the states are in the window (outside_window: no NaN, nothing beyond FP32's
+// range), and it returns false, writing nothing, where the double words would lose
+// more than FP64 does, and the caller takes the edge in FP64:
 //  - an average whose c^2 is a small difference, (H - q^2/2) < H/4 (Mach numbers
 //    above sqrt(6 / (gamma - 1)), 3.9 for gamma = 1.4), costs the double words
 //    log2(H / (H - q^2/2)) of their 48 bits (measured on the flux itself against
@@ -163,7 +164,7 @@ __device__ __forceinline__ bool edge_flux_dw_body(const EdgeArgs &A, const int64
     RoeN C;
     {
         const d4v qa = ldd4(A.Q, s[2]), qb = ldd4(A.Q, s[3]);
-        const dw4 q = d2dw4(d4v{qa.x + qb.x, qa.y + qb.y, qa.z + qb.z, qa.w + qb.w});
+        const dw4 q = d2dw4<GUARD>(d4v{qa.x + qb.x, qa.y + qb.y, qa.z + qb.z, qa.w + qb.w});
         const dw inv = norm(lrecip(q.x));
         dw mn, mt;
         turn(nx, ny, q.y, q.z, mn, mt);
@@ -175,7 +176,7 @@ __device__ __forceinline__ bool edge_flux_dw_body(const EdgeArgs &A, const int64
         // FP64 differences, then double words in the edge's frame and their
         // characteristic components: (L2-L1, R2-R1) and (L3-L1, R3-R1) paired, R1-L1
         const d4v L1 = ldd4(w, s[2]), R1 = ldd4(w, s[3]);
-        auto diff = [](const d4v &p, const d4v &q) { return d2dw4(d4v{p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w}); };
+        auto diff = [](const d4v &p, const d4v &q) { return d2dw4<GUARD>(d4v{p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w}); };
         auto two = [&](int il, int ir, int slot) {
             const dw4 l = diff(ldd4(w, il), L1), r = diff(ldd4(w, ir), R1);
             vec4<f2> d;
@@ -190,7 +191,7 @@ __device__ __forceinline__ bool edge_flux_dw_body(const EdgeArgs &A, const int64
         };
         two(s[1], s[4], 0);
         two(s[0], s[5], 4);
-        const dw4 m = diff(R1, L1), l = d2dw4(L1);
+        const dw4 m = diff(R1, L1), l = d2dw4<GUARD>(L1);
         vec4<float> d;
         d.x = m.x;
         d.w = m.w;
@@ -251,7 +252,7 @@ __device__ __forceinline__ bool edge_flux_dw_body(const EdgeArgs &A, const int64
     bool fell_back = false;
     if (!sides()) {  // positivity fallback: first-order end states
         const d4v L1 = ldd4(w, s[2]), R1 = ldd4(w, s[3]);
-        const dw4 m = d2dw4(d4v{R1.x - L1.x, R1.y - L1.y, R1.z - L1.z, R1.w - L1.w});
+        const dw4 m = d2dw4<GUARD>(d4v{R1.x - L1.x, R1.y - L1.y, R1.z - L1.z, R1.w - L1.w});
         const dw z = dw_make(0.0f);
         dw n, t;
         turn(nx, ny, m.y, m.z, n, t);

@@ -32,7 +32,10 @@ __device__ __forceinline__ d4v ldd4(const double *p, int64_t i) {
     return d4v{a.x, a.y, b.x, b.y};
 }
 
-__device__ __forceinline__ dw4 d2dw4(const d4v &v) { return d4(d2dw(v.x), d2dw(v.y), d2dw(v.z), d2dw(v.w)); }
+template <bool BOUNDED = false>
+__device__ __forceinline__ dw4 d2dw4(const d4v &v) {
+    return d4(d2dw<BOUNDED>(v.x), d2dw<BOUNDED>(v.y), d2dw<BOUNDED>(v.z), d2dw<BOUNDED>(v.w));
+}
 
 }  // namespace dwa
 }  // namespace fdu
