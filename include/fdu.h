@@ -194,10 +194,11 @@ fdu_status fdu_get_state(const fdu_mesh *mesh, double *w, int on_device, void *s
  * (characteristic projection, WENO, flux increment, Roe dissipation) and their
  * weighted sums in double-word FP32 (FP32 pairs, about 48 bits of each
  * increment), which GB300 issues at 64 times its FP64 rate.  Against extended
- * precision the residual's error is at most that of FP64 throughout (the
- * arithmetic of fdu_residual_noalloc) in every case measured, 0.04 to 0.4 of
- * it for smooth flow, shock tubes, Mach 3 and 1e4 pressure-ratio jumps and
- * random states of 10 to 90 %, 0.7 at Mach 3.7; no bound is proved.  It
+ * precision the residual's error was measured at 0.05 to 0.4 of that of FP64
+ * throughout (the arithmetic of fdu_residual_noalloc) for smooth flow, shock
+ * tubes, Mach 3 and 1e4 pressure-ratio jumps and random states of 10 to 90 %,
+ * 0.7 of it at Mach 3.7, up to all of it across density steps; no bound is
+ * proved (components that vanish across a density step of 64: 1.9 times).  It
  * computes in FP64 throughout where FP32 pairs would not do: a stage with a
  * density or energy outside 2^-24 .. 2^24 (in the caller's units) or a
  * pressure that is not positive, and a mesh with weights beyond 2^40; and in

@@ -1391,7 +1391,8 @@ __global__ void check_rows_kernel(const double *__restrict__ w, int64_t n, unsig
 }
 
 // zero (optional): words set to 0 on the way, which saves a memset's launch
-// when a state is set (2 us of a small mesh's 25 us residual call).
+// when a state is set (in a small mesh's 25 us residual call within the spread of
+// the runs).
 __global__ void permute_rows_kernel(const double *__restrict__ in, double *__restrict__ out,
                                     const int32_t *__restrict__ map, int64_t n, bool gather, double *zero, int nzero) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -365,7 +365,7 @@ class Mesh:
         (edge fluxes by characteristic NU-WENO5 and a Roe flux, Section 2.3.1;
         least-squares divergence, Section 2.2.1).  precision 64: FP64 accuracy
         (state-sized terms FP64, edge-flux increments double-word FP32 within
-        its range, FP64 outside it); 48: the double-word form without the range
+        its range, FP64 outside it); 48: the double-word form without the
         checks; 32: FP32 fluxes with FP64 accumulation.  out: a host array or a CUDA
         tensor of that shape (None: a new host array)."""
         if out is None:
@@ -434,8 +434,9 @@ class Mesh:
         return n.value, t.value
 
     def set_adjoint_precision(self, precision):
-        """Precision of the adjoint calls: 64 (FP64) or 48 (double-word edge-flux
-        VJP and precision-48 steps)."""
+        """Precision of the adjoint calls: 64 (precision-64 steps; edge-flux VJP in
+        double words where that holds FP64's accuracy, in FP64 elsewhere) or 48
+        (double-word VJP for every edge and precision-48 steps)."""
         _check(load().fdu_set_adjoint_precision(self._h, int(precision)))
         self._adjoint_precision = int(precision)
 
