@@ -286,13 +286,14 @@ __device__ __forceinline__ double scaled_down(double x, int k) {
     return __hiloint2double((__double2hiint(x) & (int)0x800fffff) | (e << 20), __double2loint(x));
 }
 
-// GUARD (precision 64): returns false for an edge that FP64 takes and writes: a state outside the forward kernel's density and energy window,
-// differences that are not finite in FP32 (a NaN or huge momentum), an average whose c^2 is a
-// small difference (edge_flux_dw_body), a cotangent that is not finite, or a
-// WENO epsilon so far below the state's squares that the derivative of the
-// weights rests on the rounding of the differences (eps < 2^-76 max(rho, E)^2:
-// noise of 2^-53 of the state, squared, would pass for an indicator; the fields
-// are in units of density and momentum, |m|^2 < 2 rho E), or end states more
+// GUARD (precision 64): returns false for an edge that FP64 takes and writes: a
+// state outside the forward kernel's density and energy window, differences that
+// are not finite in FP32 (a NaN or huge momentum), an average whose c^2 is a small
+// difference (edge_flux_dw_body), a cotangent that is not finite, a WENO epsilon so
+// far below the state's squares that the derivative of the weights rests on the
+// rounding of the differences (eps < 2^-76 max(rho, E)^2: noise of 2^-53 of the
+// state, squared, would pass for an indicator; the fields are in units of density
+// and momentum, |m|^2 < 2 rho E), outputs beyond FP32's range, or end states more
 // than a factor of two apart in density or energy.  VJP against central
 // differences in extended precision, FP64 / double words without the last line /
 // with it, steps of 4, 16, 64 in density and pressure: 7.7e-14 / 1.4e-13 / 3.1e-14,

@@ -150,6 +150,7 @@ struct fdu_mesh {
             no_memory = e == cudaErrorMemoryAllocation;
             return set_err(FDU_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
         }
+        no_memory = false;
         allocs.push_back(q);
         device_bytes += (int64_t)bytes;
         return FDU_OK;
